@@ -27,6 +27,8 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "cover.cuh"
+#include "rowlists.cuh"
 
 namespace tcgs {
 namespace {
@@ -70,35 +72,6 @@ __device__ __forceinline__ uint32_t warp_peers(uint32_t v, bool valid) {
         peers &= bit ? bal : ~bal;
     }
     return peers;
-}
-
-// Exclusive scan over a block of NT threads; returns the thread's exclusive prefix and the total.
-template <typename T, int NT>
-__device__ __forceinline__ T block_exclusive_scan(T x, T* warp_sums, T& total) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    T v = x;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        T y = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += y;
-    }
-    if (lane == 31) warp_sums[warp] = v;
-    __syncthreads();
-    if (warp == 0) {
-        constexpr int NW = NT / 32;
-        T w = lane < NW ? warp_sums[lane] : T(0);
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            T y = __shfl_up_sync(0xffffffffu, w, o);
-            if (lane >= o) w += y;
-        }
-        if (lane < NW) warp_sums[lane] = w;
-    }
-    __syncthreads();
-    T before = warp > 0 ? warp_sums[warp - 1] : T(0);
-    total = warp_sums[NT / 32 - 1];
-    __syncthreads();
-    return before + v - x;
 }
 
 // ---------------------------------------------------------------- radix sort passes
@@ -337,38 +310,6 @@ __global__ void __launch_bounds__(kThreads) k_radix_scatter(const uint32_t* __re
 
 // ---------------------------------------------------------------- binning kernels
 
-__device__ __forceinline__ uint32_t orderable_bits(float f) {
-    uint32_t u = __float_as_uint(f);
-    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-}
-
-// Exact tile coverage (tcgs_bin_sort_exact): Gaussian g reaches tile t when the least value of its
-// conic form over t's 16 x 16 box of pixel centres, in tile-local coordinates, is at most its reach
-// limit (the TC renderer's block-mark limit, whose boxes lie inside the tile's).  Per warp, the 32
-// Gaussians' parameters are staged in shared memory once; every splat then reads its Gaussian's.
-struct Cover {
-    float mx, my, a, b, c, ia, ic, lim;
-};
-
-__device__ __forceinline__ Cover cover_of(const float* __restrict__ mean2d, const float* __restrict__ conic,
-                                          const float* __restrict__ opacity, uint32_t g) {
-    Cover v;
-    const float2 m = reinterpret_cast<const float2*>(mean2d)[g];
-    v.mx = m.x; v.my = m.y;
-    v.a = conic[3 * g]; v.b = conic[3 * g + 1]; v.c = conic[3 * g + 2];
-    v.lim = reach_limit(__logf(opacity[g]));
-    v.ia = __fdividef(1.f, v.a);
-    v.ic = __fdividef(1.f, v.c);
-    return v;
-}
-
-// Gaussian v reaches the tile whose centre is at tile-local offset (lx, ly) from its mean when the
-// least value of its conic form over the tile's 16 x 16 pixel-centre box is within its reach limit.
-__device__ __forceinline__ bool tile_reached(const Cover& v, float lx, float ly) {
-    constexpr float h = 0.5f * (kTile - 1);
-    return v.lim >= 0.f && min_q_box_facing(lx, ly, v.a, v.b, v.c, v.ia, v.ic, -h, h, -h, h) <= v.lim;
-}
-
 // Row and column of tile kk of a rectangle `w` tiles wide: the quotient from a float product and one
 // correction step (exact for kk < 2^22: the product is then within one of kk / w), integer division
 // beyond that.
@@ -475,108 +416,6 @@ __device__ __forceinline__ void block_cover_splats(BlockCover& bc, uint32_t grid
     }
 }
 
-// ---- exact coverage by tile rows
-//
-// In one row of tiles the tiles a Gaussian reaches form an interval: their pixel-centre boxes span
-// the same band of rows, and a box meets the convex region {q <= lim} exactly when its x-range meets
-// the region's shadow on the x axis within that band.  So each (Gaussian, tile row) is one unit of
-// work: the shadow's ends come from the ellipse in closed form, and the per-tile test (tile_reached)
-// fixes the interval's end tiles, so the tiles kept are those the per-tile test keeps (whenever they
-// form one run, which they do up to FP32 ties at the reach limit).  Narrow rows and degenerate
-// conics test every tile of the row and keep the run from the first to the last passing tile.
-
-// Extent of the reach ellipse {q <= lim} about the mean: half-widths W (x) and H (y), the y offset s
-// of its leftmost point (the rightmost one is at -s), and det = ac - b^2.  W < 0: scan the row.
-struct Reach {
-    float W, H, s, det;
-};
-
-__device__ __forceinline__ Reach reach_of(const Cover& v) {
-    Reach e;
-    e.det = __fsub_rn(__fmul_rn(v.a, v.c), __fmul_rn(v.b, v.b));
-    e.W = -1.f;
-    e.H = e.s = 0.f;
-    if (!(e.det > 0.f) || !(v.lim >= 0.f)) return e;
-    const float idet = __frcp_rn(e.det);
-    const float W = __fsqrt_rn(__fmul_rn(__fmul_rn(v.lim, v.c), idet));
-    const float H = __fsqrt_rn(__fmul_rn(__fmul_rn(v.lim, v.a), idet));
-    if (!(W < 1e30f) || !(H < 1e30f)) return e;
-    e.W = W;
-    e.H = H;
-    e.s = __fmul_rn(__fmul_rn(v.b, W), v.ic);
-    return e;
-}
-
-__device__ __forceinline__ int clamp_tile(float f, int lo, int hi) {
-    return (int)fminf(fmaxf(f, (float)lo), (float)hi);   // NaN -> lo
-}
-
-// Tiles [L, R] (empty when L > R) of rectangle columns [x0, x1] in tile row ty that Gaussian v reaches.
-__device__ int2 row_span(const Cover& v, const Reach& e, int ty, int x0, int x1) {
-    const int2 none = make_int2(1, 0);
-    if (!(v.lim >= 0.f)) return none;
-    const float ly = v.my - (float)(ty * kTile + kTile / 2);
-    auto test = [&](int tx) { return tile_reached(v, v.mx - (float)(tx * kTile + kTile / 2), ly); };
-    auto scan = [&]() {
-        int L = x0;
-        while (L <= x1 && !test(L)) ++L;
-        if (L > x1) return none;
-        int R = x1;
-        while (R > L && !test(R)) --R;
-        return make_int2(L, R);
-    };
-    if (e.W < 0.f || x1 - x0 < 3) return scan();
-    // the shadow [xa, xb] of the ellipse on the x axis within the row's band of pixel centres
-    const float yl = __fsub_rn((float)(ty * kTile) + 0.5f, v.my), yh = __fadd_rn(yl, 15.f);
-    float Lf = 1.f, Rf = 0.f;   // empty unless the band meets the ellipse
-    if (!(yl > e.H || yh < -e.H)) {
-        const float alim = __fmul_rn(v.a, v.lim);
-        const float dl = fminf(yh, fmaxf(yl, e.s)), dr = fminf(yh, fmaxf(yl, -e.s));
-        const float rl = __fsqrt_rn(fmaxf(0.f, __fsub_rn(alim, __fmul_rn(e.det, __fmul_rn(dl, dl)))));
-        const float rr = __fsqrt_rn(fmaxf(0.f, __fsub_rn(alim, __fmul_rn(e.det, __fmul_rn(dr, dr)))));
-        const float xa = __fmul_rn(__fsub_rn(__fmul_rn(-v.b, dl), rl), v.ia);
-        const float xb = __fmul_rn(__fadd_rn(__fmul_rn(-v.b, dr), rr), v.ia);
-        // tiles whose box [16 tx + 0.5, 16 tx + 15.5] meets [mx + xa, mx + xb]
-        Lf = ceilf(__fmul_rn(__fsub_rn(__fadd_rn(v.mx, xa), 15.5f), 1.f / kTile));
-        Rf = floorf(__fmul_rn(__fsub_rn(__fadd_rn(v.mx, xb), 0.5f), 1.f / kTile));
-    }
-    if (!(Lf <= Rf) || Rf < (float)x0 || Lf > (float)x1) {
-        // no shadow in the rectangle: probe the tile holding the point of least q in the band (the
-        // least of the minima over x, (det / a) dy^2, is at the dy nearest to 0), grow from there
-        const float dyc = fminf(yh, fmaxf(yl, 0.f));
-        const float xc = __fadd_rn(v.mx, __fmul_rn(__fmul_rn(-v.b, dyc), v.ia));
-        const int c = clamp_tile(floorf(__fmul_rn(xc, 1.f / kTile)), x0, x1);
-        if (!test(c)) return none;
-        int L = c, R = c;
-        while (L > x0 && test(L - 1)) --L;
-        while (R < x1 && test(R + 1)) ++R;
-        return make_int2(L, R);
-    }
-    int L = clamp_tile(Lf, x0, x1), R = clamp_tile(Rf, x0, x1);
-    if (test(L)) {
-        while (L > x0 && test(L - 1)) --L;
-    } else {
-        int k = L + 1;
-        while (k <= R && !test(k)) ++k;
-        if (k > R) return scan();
-        L = k;
-    }
-    if (test(R)) {
-        while (R < x1 && test(R + 1)) ++R;
-    } else {
-        int k = R - 1;
-        while (k > L && !test(k)) --k;
-        R = k;
-    }
-    return make_int2(L, R);
-}
-
-// Gaussians whose rectangle is at least this many tiles wide are covered by rows; the narrower ones
-// tile by tile (for them a row costs about as many box tests as it has tiles, plus the row's own
-// bookkeeping).
-constexpr int kRowMinWidth = 6;
-// The row path runs when the caller's splat capacity allows at least this many splats per Gaussian.
-constexpr int kRowsCapacityPerGaussian = 32;
 // The packed tile sort runs for capacities of at least this many splats: on short lists it gains
 // nothing (bin_sort of the 2.3M-splat 1080p frame 0.226 ms either way; 11.6M splats 0.527 -> 0.491 ms;
 // 605M splats 15.8 -> 12.7 ms).
@@ -1177,6 +1016,19 @@ extern "C" size_t tcgs_bin_sort_workspace_size(int32_t P, int64_t splat_capacity
 namespace tcgs {
 namespace {
 
+// The depth order of the P keys and indices in the a-buffers, back in them (4 passes); returns the
+// number of passes.
+int depth_order(const Workspace& w, uint32_t P, cudaStream_t s) {
+    const int G = sort_blocks<kItems>(P);
+    int pass = 0;
+    for (int sh = 0; sh < 32; sh += 8, ++pass) {
+        const bool even = (pass & 1) == 0;
+        radix_pass<kItems>(even ? w.dk_a : w.dk_b, even ? w.dv_a : w.dv_b, even ? w.dk_b : w.dk_a,
+                           even ? w.dv_b : w.dv_a, P, nullptr, sh, 8, G, w, pass, s);
+    }
+    return pass;
+}
+
 // The sorting stage; `exact` selects the exact tile coverage (conic and opacity are then read).
 tcgs_status bin_sort(const tcgs_camera* cam, int32_t P, const float* mean2d, const int32_t* radius,
                      const float* depth, bool exact, const float* conic, const float* opacity,
@@ -1194,13 +1046,28 @@ tcgs_status bin_sort(const tcgs_camera* cam, int32_t P, const float* mean2d, con
     Workspace w = layout((char*)workspace, P, splat_capacity);
     if (ws_bytes < w.bytes) return TCGS_ERR_INVALID;
 
+    const bool small = P <= kSmallMaxP && splat_capacity <= kSmallMaxCapacity && num_tiles <= kSmallMaxTiles;
+    // the coverage of wide Gaussians by rows pays off for wide footprints: chosen when the caller's capacity
+    // allows at least kRowsCapacityPerGaussian splats per Gaussian (the lists are the same either way)
+    const bool rows = exact && splat_capacity >= (int64_t)kRowsCapacityPerGaussian * P;
+    if (!small && P > 0 && dc.grid_w <= kRowListsMaxGrid && dc.grid_h <= kRowListsMaxGrid) {
+        // depth order, then lists by tile rows (in the workspace from the counts on: the depth passes'
+        // histograms there are done with by then)
+        RowLists a{dc, (uint32_t)P, w.dv_a, mean2d, radius, conic, opacity, exact, rows, splat_capacity,
+                   (char*)w.counts, ids_sorted, tile_ranges, n_splats, status};
+        if ((size_t)(a.scratch - (char*)workspace) + row_lists_scratch_bytes(P, splat_capacity) > w.bytes)
+            return TCGS_ERR_INVALID;   // never: the splat buffers hold the runs
+        launch_row_keys(a, depth, w.dk_a, w.dv_a, w.digit_total, s);
+        depth_order(w, (uint32_t)P, s);
+        launch_row_lists(a, s);
+        TCGS_CHECK_LAUNCH();
+        return TCGS_OK;
+    }
+
     // keys, counts, range clearing, digit totals of pass 0
     int n_init = P > 2 * num_tiles ? P : 2 * num_tiles;
     if (n_init < kThreads) n_init = kThreads;
     const int kb_blocks = (n_init + kThreads - 1) / kThreads;
-    // the row path pays off for wide footprints: chosen when the caller's capacity allows at least
-    // kRowsCapacityPerGaussian splats per Gaussian (the lists are the same either way)
-    const bool rows = exact && splat_capacity >= (int64_t)kRowsCapacityPerGaussian * P;
     if (rows)
         launch_pdl(k_bin_keys<true, true>, kb_blocks, kThreads, 0, s, dc, P, mean2d, radius, depth, conic, opacity, w.dk_a,
                    w.dv_a, w.counts, tile_ranges, 2 * num_tiles, w.digit_total);
@@ -1212,7 +1079,6 @@ tcgs_status bin_sort(const tcgs_camera* cam, int32_t P, const float* mean2d, con
                    w.dv_a, w.counts, tile_ranges, 2 * num_tiles, w.digit_total);
     count_launches(1);
     TCGS_CHECK_LAUNCH();
-    const bool small = P <= kSmallMaxP && splat_capacity <= kSmallMaxCapacity && num_tiles <= kSmallMaxTiles;
     if (small) {
         // 1-2 in one CTA
         launch_pdl(k_small_depth_scan, 1, kSmallThreads, 0, s, (uint32_t)P, w.dk_a, w.dv_a, w.dk_b, w.dv_b, w.counts,
@@ -1241,12 +1107,7 @@ tcgs_status bin_sort(const tcgs_camera* cam, int32_t P, const float* mean2d, con
     // 1. depth order (4 passes; the result returns to the a-buffers)
     int pass = 0;
     if (P > 0) {
-        int Gp = sort_blocks<kItems>(P);
-        for (int sh = 0; sh < 32; sh += 8, ++pass) {
-            bool even = (pass & 1) == 0;
-            radix_pass<kItems>(even ? w.dk_a : w.dk_b, even ? w.dv_a : w.dv_b, even ? w.dk_b : w.dk_a,
-                       even ? w.dv_b : w.dv_a, (uint32_t)P, nullptr, sh, 8, Gp, w, pass, s);
-        }
+        pass = depth_order(w, (uint32_t)P, s);
         TCGS_CHECK_LAUNCH();
     }
     const uint32_t* order = w.dv_a;
