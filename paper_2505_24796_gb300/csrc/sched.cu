@@ -7,7 +7,7 @@
 // queue is ordered longest-predicted first.  Its training data are the per-tile costs the
 // renderer itself records (tile_stats).
 //
-// Kernels: per-tile features (one warp per tile), feature normaliser, MLP forward, MLP backward
+// Kernels: per-tile features (one block per tile), feature normaliser, MLP forward, MLP backward
 // (mean squared error), Adam.  The ordering sort lives with the radix sort in binsort.cu.
 #include "common.cuh"
 
@@ -24,48 +24,88 @@ __device__ __forceinline__ float h16(float x) { return __half2float(__float2half
 
 // ---------------------------------------------------------------- features
 
-__global__ void __launch_bounds__(256) k_tile_features(DevCamera cam, const uint32_t* __restrict__ ranges,
-                                                       const uint32_t* __restrict__ ids,
-                                                       const float* __restrict__ mean2d,
-                                                       const float* __restrict__ conic,
-                                                       const float* __restrict__ opacity,
-                                                       const float* __restrict__ depth,
-                                                       const int32_t* __restrict__ radius, float* __restrict__ feat) {
-    const int tiles = cam.grid_w * cam.grid_h;
-    const int tile = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (tile >= tiles) return;
+constexpr int kFewTilesPerSm = 4;
+
+// One block of NT threads per tile.  Bound by the latency of two dependent gathers (id, then the
+// Gaussian's values from L2) on lists of thousands of entries, so a tile gets as many threads as keep
+// enough of them in flight: 16 views of 320 x 240 (300 tiles each, about 8000 entries a tile) took 8.13 ms
+// with one warp a tile and take 0.79 ms, which is about the sectors the gathers touch in L2 (six a list entry).
+template <int NT>
+__global__ void __launch_bounds__(NT) k_tile_features(DevCamera cam, const uint32_t* __restrict__ ranges,
+                                                      const uint32_t* __restrict__ ids,
+                                                      const float* __restrict__ mean2d,
+                                                      const float* __restrict__ conic,
+                                                      const float* __restrict__ opacity,
+                                                      const float* __restrict__ depth,
+                                                      const int32_t* __restrict__ radius, float* __restrict__ feat) {
+    constexpr int kSums = 6, kDeep = 4;   // entries a thread has in flight
+    __shared__ float s_sum[NT / 32][kSums];
+    const int tile = blockIdx.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int tx = tile % cam.grid_w, ty = tile / cam.grid_w;
     const float x0 = (float)(kTile * tx), y0 = (float)(kTile * ty);
-    const uint32_t start = ranges[2 * tile], end = ranges[2 * tile + 1];
+    const uint32_t start = ranges[2 * tile], end = ranges[2 * tile + 1], len = end - start;
     float so = 0.f, mo = 0.f, dmin = 3.0e38f, dmax = -3.0e38f, sdet = 0.f, cov = 0.f;
-    for (uint32_t i = start + lane; i < end; i += 32) {
-        const uint32_t g = ids[i];
-        const float o = opacity[g];
-        so += o;
-        mo = fmaxf(mo, o);
-        const float d = depth[g];
-        dmin = fminf(dmin, d);
-        dmax = fmaxf(dmax, d);
-        const float a = conic[3 * g], b = conic[3 * g + 1], c = conic[3 * g + 2];
-        sdet += __logf(fmaxf(a * c - b * b, 1e-30f));
-        const float2 m = reinterpret_cast<const float2*>(mean2d)[g];
-        const float r = (float)radius[g];
-        const float ox = fmaxf(0.f, fminf(m.x + r, x0 + kTile) - fmaxf(m.x - r, x0));
-        const float oy = fmaxf(0.f, fminf(m.y + r, y0 + kTile) - fmaxf(m.y - r, y0));
-        cov += ox * oy * (1.f / (kTile * kTile));
-    }
+    for (uint32_t k0 = threadIdx.x; k0 < len; k0 += kDeep * NT) {
+        uint32_t g[kDeep];
+        bool in[kDeep];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        so += __shfl_xor_sync(0xffffffffu, so, o);
-        mo = fmaxf(mo, __shfl_xor_sync(0xffffffffu, mo, o));
-        dmin = fminf(dmin, __shfl_xor_sync(0xffffffffu, dmin, o));
-        dmax = fmaxf(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
-        sdet += __shfl_xor_sync(0xffffffffu, sdet, o);
-        cov += __shfl_xor_sync(0xffffffffu, cov, o);
+        for (int u = 0; u < kDeep; ++u) {
+            in[u] = k0 + u * NT < len;
+            g[u] = ids[start + (in[u] ? k0 + u * NT : k0)];
+        }
+        float o[kDeep], d[kDeep], a[kDeep], b[kDeep], c[kDeep], r[kDeep];
+        float2 m[kDeep];
+#pragma unroll
+        for (int u = 0; u < kDeep; ++u) {
+            o[u] = opacity[g[u]];
+            d[u] = depth[g[u]];
+            a[u] = conic[3 * g[u]]; b[u] = conic[3 * g[u] + 1]; c[u] = conic[3 * g[u] + 2];
+            m[u] = reinterpret_cast<const float2*>(mean2d)[g[u]];
+            r[u] = (float)radius[g[u]];
+        }
+#pragma unroll
+        for (int u = 0; u < kDeep; ++u) {
+            if (!in[u]) continue;
+            so += o[u];
+            mo = fmaxf(mo, o[u]);
+            dmin = fminf(dmin, d[u]);
+            dmax = fmaxf(dmax, d[u]);
+            sdet += __logf(fmaxf(a[u] * c[u] - b[u] * b[u], 1e-30f));
+            const float ox = fmaxf(0.f, fminf(m[u].x + r[u], x0 + kTile) - fmaxf(m[u].x - r[u], x0));
+            const float oy = fmaxf(0.f, fminf(m[u].y + r[u], y0 + kTile) - fmaxf(m[u].y - r[u], y0));
+            cov += ox * oy * (1.f / (kTile * kTile));
+        }
     }
+    auto over_warp = [&]() {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            so += __shfl_xor_sync(0xffffffffu, so, o);
+            mo = fmaxf(mo, __shfl_xor_sync(0xffffffffu, mo, o));
+            dmin = fminf(dmin, __shfl_xor_sync(0xffffffffu, dmin, o));
+            dmax = fmaxf(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
+            sdet += __shfl_xor_sync(0xffffffffu, sdet, o);
+            cov += __shfl_xor_sync(0xffffffffu, cov, o);
+        }
+    };
+    over_warp();
     if (lane == 0) {
-        const float n = (float)(end - start);
+        const float v[kSums] = {so, mo, dmin, dmax, sdet, cov};
+#pragma unroll
+        for (int k = 0; k < kSums; ++k) s_sum[warp][k] = v[k];
+    }
+    __syncthreads();
+    if (warp > 0) return;
+    const bool in = lane < NT / 32;
+    so = in ? s_sum[lane][0] : 0.f;
+    mo = in ? s_sum[lane][1] : 0.f;
+    dmin = in ? s_sum[lane][2] : 3.0e38f;
+    dmax = in ? s_sum[lane][3] : -3.0e38f;
+    sdet = in ? s_sum[lane][4] : 0.f;
+    cov = in ? s_sum[lane][5] : 0.f;
+    over_warp();
+    if (lane == 0) {
+        const float n = (float)len;
         const float inv = n > 0.f ? 1.f / n : 0.f;
         const int w_in = min(kTile, cam.width - kTile * tx), h_in = min(kTile, cam.height - kTile * ty);
         float* f = feat + (size_t)tile * kIn;
@@ -261,8 +301,15 @@ extern "C" tcgs_status tcgs_tile_features(const tcgs_camera* cam, const uint32_t
         return TCGS_ERR_INVALID;
     const DevCamera dc = make_dev_camera(*cam);
     const int tiles = dc.grid_w * dc.grid_h;
-    k_tile_features<<<(tiles * 32 + 255) / 256, 256, 0, (cudaStream_t)stream>>>(dc, tile_ranges, ids_sorted, mean2d,
-                                                                              conic, opacity, depth, radius, features);
+    // a view of few tiles leaves most of the chip idle unless each tile gets many warps
+    DeviceInfo d;
+    const int sms = current_device_info(&d) ? d.sms : 128;
+    if (tiles <= kFewTilesPerSm * sms)
+        k_tile_features<512><<<tiles, 512, 0, (cudaStream_t)stream>>>(dc, tile_ranges, ids_sorted, mean2d, conic, opacity,
+                                                                      depth, radius, features);
+    else
+        k_tile_features<128><<<tiles, 128, 0, (cudaStream_t)stream>>>(dc, tile_ranges, ids_sorted, mean2d, conic, opacity,
+                                                                      depth, radius, features);
     count_launches(1);
     TCGS_CHECK_LAUNCH();
     return TCGS_OK;

@@ -1,0 +1,45 @@
+"""Kernels at the edges of their blocks, batches and dispatch rules, against the FP64 oracle."""
+import numpy as np
+import pytest
+
+import oracle
+from oracle import sched as osc
+from paper_2505_24796_gb300 import scenes
+
+from .helpers import f32, to_torch
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+@pytest.fixture(scope="module")
+def tc():
+    import paper_2505_24796_gb300 as m
+    m._lib.load()
+    return m
+
+
+@pytest.mark.parametrize("width,height", [(60, 40), (800, 400)])
+def test_tile_features_list_lengths(tc, width, height):
+    """Lists around the multiples of a block's threads and of its entries in flight, in a view of few tiles
+    (512 threads a tile) and one of many (128).  FP32 sums of at most 2049 terms: 1e-4 as for the
+    workload's lists."""
+    cam = scenes.pinhole(width, height, fx=100.0)
+    gw, gh = oracle.grid(cam)
+    rng = np.random.default_rng(3)
+    P = 4000
+    lens = np.resize([0, 1, 31, 127, 128, 129, 511, 512, 513, 2047, 2048, 2049], gw * gh)
+    ends = np.cumsum(lens)
+    a, c = rng.uniform(0.05, 1.0, (2, P))
+    inp = dict(mean2d=f32(rng.uniform(0, width, (P, 2))),
+               conic=f32(np.stack([a, 0.9 * rng.uniform(-1, 1, P) * np.sqrt(a * c), c], 1)),
+               opacity=f32(rng.uniform(0.01, 1, P)), depth=f32(rng.uniform(1, 9, P)),
+               radius=rng.integers(1, 30, P).astype(np.int32))
+    b = dict(ids=rng.integers(0, P, int(ends[-1])), ranges=np.stack([ends - lens, ends], 1), n=int(ends[-1]))
+    ref = osc.tile_features(cam, b, inp["mean2d"], inp["conic"], inp["opacity"], inp["depth"], inp["radius"])
+    d = {k: to_torch(v, DEV) for k, v in inp.items()}
+    got = tc.tcgs_tile_features(cam, to_torch(b["ranges"].astype(np.int32), DEV), to_torch(b["ids"].astype(np.int32), DEV),
+                                d["mean2d"], d["conic"], d["opacity"], d["depth"], d["radius"])
+    torch.cuda.synchronize()
+    np.testing.assert_allclose(got.cpu().numpy(), ref, rtol=1e-4, atol=1e-4)
