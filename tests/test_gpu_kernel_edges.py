@@ -43,3 +43,25 @@ def test_tile_features_list_lengths(tc, width, height):
                                 d["mean2d"], d["conic"], d["opacity"], d["depth"], d["radius"])
     torch.cuda.synchronize()
     np.testing.assert_allclose(got.cpu().numpy(), ref, rtol=1e-4, atol=1e-4)
+
+
+@pytest.mark.parametrize("n", [1, 31, 127, 128, 129, 300])
+def test_mlp_block_edges(tc, n):
+    """Item counts around the block's 128.  The targets lie 2 to 4 from the outputs, so that an FP16 rounding
+    that falls the other way (2e-3 (1 + |y|) of the output, as in the workload's test) moves a gradient by
+    at most about 0.5% of the largest."""
+    rng = np.random.default_rng(n)
+    p = osc.unpack(rng.normal(0, 0.3, osc.NPARAMS))
+    p["b1"], p["b2"] = np.abs(p["b1"]) + 0.05, np.abs(p["b2"]) + 0.05
+    params, X = f32(osc.pack(p)), f32(rng.normal(0, 2, (n, 8)) + 1.0)
+    norm = f32(np.concatenate([np.full(8, 1.0), np.full(8, 0.5)]))
+    yr, _ = osc.mlp_forward(params.astype(np.float64), norm.astype(np.float64), X, fp16=True)
+    t = f32(yr + rng.uniform(2, 4, n) * rng.choice([-1, 1], n))
+    d = [to_torch(v, DEV) for v in (params, norm, X)]
+    y = tc.tcgs_mlp_fwd(*d).cpu().numpy()
+    assert (np.abs(y - yr) <= 2e-3 * (1 + np.abs(yr))).all()
+    loss = torch.zeros(1, device=DEV)
+    grad, _ = tc.tcgs_mlp_bwd(*d, to_torch(t, DEV), loss=loss)
+    gr, lr = osc.mlp_backward(params.astype(np.float64), norm.astype(np.float64), X, t, fp16=True)
+    assert np.abs(grad.cpu().numpy() - gr).max() <= 1e-2 * np.abs(gr).max()
+    assert abs(float(loss.item()) - lr) <= 1e-2 * lr
