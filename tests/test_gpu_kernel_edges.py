@@ -6,7 +6,7 @@ import oracle
 from oracle import sched as osc
 from paper_2505_24796_gb300 import scenes
 
-from .helpers import f32, to_torch
+from .helpers import f32, scene64, to_torch
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -65,3 +65,46 @@ def test_mlp_block_edges(tc, n):
     gr, lr = osc.mlp_backward(params.astype(np.float64), norm.astype(np.float64), X, t, fp16=True)
     assert np.abs(grad.cpu().numpy() - gr).max() <= 1e-2 * np.abs(gr).max()
     assert abs(float(loss.item()) - lr) <= 1e-2 * lr
+
+
+@pytest.mark.parametrize("aligned", [True, False])
+@pytest.mark.parametrize("degree", [0, 1, 2, 3])
+def test_project_backward_rows_and_alignment(tc, degree, aligned):
+    """Gaussian counts around a warp's 32 rows and a block's 128, every SH degree, coefficient arrays on and off
+    a 16-byte boundary: the oracle's gradients (bounds as for the workloads), rows of unseen Gaussians
+    untouched, and a second call adds the same again."""
+    for P in (1, 31, 32, 33, 127, 161):
+        cam, sc = scenes.plain_forward(P=P, seed=40 + P)
+        rng = np.random.default_rng(P)
+        K = (degree + 1) ** 2
+        sc = dict(sc, sh=f32(rng.normal(0, 0.3, (P, K, 3))), sh_degree=degree)
+        sc["means3"] = sc["means3"].copy()
+        sc["means3"][::5, 2] = -1.0     # behind the camera
+        pr = oracle.project(cam, scene64(sc))
+        w = [f32(rng.normal(size=(P, k))) for k in (2, 3, 3)]
+        ref = oracle.project_bwd(cam, scene64(sc), pr["radius"], *w)
+        off = 0 if aligned else 1
+
+        def place(a):
+            buf = torch.zeros(a.size + off, device=DEV)
+            v = buf[off:].view(a.shape)
+            v.copy_(torch.from_numpy(a))
+            return v
+
+        d = tc.scene_to_device(sc, DEV)
+        grads = dict(dmeans3=torch.zeros(P, 3, device=DEV), dscales=torch.zeros(P, 3, device=DEV),
+                     dquats=torch.zeros(P, 4, device=DEV), dsh=place(np.zeros((P, K, 3), np.float32)))
+        args = (cam, d["means3"], d["scales"], d["quats"], place(sc["sh"]), degree,
+                to_torch(pr["radius"].astype(np.int32), DEV), *(to_torch(v, DEV) for v in w))
+        tc.tcgs_project_bwd(*args, grads=grads)
+        once = {k: v.cpu().numpy().astype(np.float64) for k, v in grads.items()}
+        tc.tcgs_project_bwd(*args, grads=grads)
+        seen = pr["radius"] > 0
+        for k, v in once.items():
+            assert (v[~seen] == 0).all()
+            np.testing.assert_allclose(grads[k].cpu().numpy(), 2 * v, rtol=1e-6, atol=0)
+            if seen.any():
+                r = ref[k].reshape(P, -1)[seen]
+                scale = np.abs(r).max(axis=1) + 1e-6 * (np.abs(r).max() + 1e-30)
+                err = np.abs(v.reshape(P, -1)[seen] - r).max(axis=1) / scale
+                assert err.max() <= 2e-3, (P, k, err.max())
