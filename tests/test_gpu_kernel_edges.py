@@ -6,7 +6,7 @@ import oracle
 from oracle import sched as osc
 from paper_2505_24796_gb300 import scenes
 
-from .helpers import f32, scene64, to_torch
+from .helpers import f32, margin_mask, scene64, to_torch
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -108,3 +108,127 @@ def test_project_backward_rows_and_alignment(tc, degree, aligned):
                 scale = np.abs(r).max(axis=1) + 1e-6 * (np.abs(r).max() + 1e-30)
                 err = np.abs(v.reshape(P, -1)[seen] - r).max(axis=1) / scale
                 assert err.max() <= 2e-3, (P, k, err.max())
+
+
+def _pair_case(rng, lens, wide):
+    """A 40 x 40 view (9 tiles) whose tiles' lists have the given lengths; wide: footprints of many tiles."""
+    cam = scenes.pinhole(40, 40, fx=50.0)
+    n = int(np.sum(lens))
+    ends = np.cumsum(lens)
+    t = np.repeat(np.arange(9), lens)
+    a, c = rng.uniform(*((0.0005, 0.005) if wide else (0.02, 1.5)), (2, n))
+    inp = dict(mean2d=f32(np.stack([t % 3 * 16 + rng.uniform(-4, 20, n), t // 3 * 16 + rng.uniform(-4, 20, n)], 1)),
+               conic=f32(np.stack([a, 0.95 * rng.uniform(-1, 1, n) * np.sqrt(a * c), c], 1)),
+               opacity=f32(rng.uniform(0.002, 0.5, n)), rgb=f32(rng.uniform(0, 1, (n, 3))))
+    b = dict(ids=np.arange(n), ranges=np.stack([ends - lens, ends], 1).astype(np.int64), n=n)
+    return cam, inp, b
+
+
+def _render(tc, cam, inp, b, bg=(0, 0, 0), **kw):
+    d = {k: to_torch(v, DEV) for k, v in inp.items()}
+    lists = (to_torch(b["ranges"].astype(np.int32), DEV), to_torch(b["ids"].astype(np.int32), DEV))
+    return d, lists, tc.tcgs_render_fwd(cam, tc.render_opts("fp32", **kw), *lists, d["mean2d"], d["conic"], d["opacity"],
+                                        d["rgb"], bg=bg)
+
+
+LENGTHS = np.array([0, 1, 3, 4, 5, 127, 128, 129, 260])   # around the group (4) and the batch (128)
+
+
+@pytest.mark.parametrize("early", [False, True])
+def test_fp32_blending_list_lengths(tc, early):
+    """Forward and backward against the oracle, a view whose last row and column of tiles are partly outside.
+    Footprints of a few pixels, whose transmittance stays above 0.05: the image to 1e-5, as for the workloads,
+    and the gradients to 2e-4 of the Gaussian's largest component + 1e-3 of the array's, as at full size."""
+    rng = np.random.default_rng(5)
+    cam, inp, b = _pair_case(rng, LENGTHS, False)
+    bg = (0.25, 0.5, 0.75)
+    d, lists, f = _render(tc, cam, inp, b, bg, early_cull=early)
+    i64 = {k: v.astype(np.float64) for k, v in inp.items()}
+    o = oracle.render(cam, b, i64["mean2d"], i64["conic"], i64["opacity"], i64["rgb"], bg=bg)
+    G = f32(rng.standard_normal((3, 40, 40)))
+    margin = margin_mask(o)
+    G[:, margin] = 0
+    assert margin.mean() < 0.01
+    assert np.abs(f["img"].cpu().numpy() - o["img"]).max(axis=0)[~margin].max() <= 1e-5
+    ref = oracle.render_bwd(cam, b, i64["mean2d"], i64["conic"], i64["opacity"], i64["rgb"], G.astype(np.float64), bg=bg)
+    g = tc.tcgs_render_bwd(cam, tc.render_opts("fp32", early_cull=early), *lists, d["mean2d"], d["conic"], d["opacity"],
+                           d["rgb"], f["img"], f["T_final"], f["n_contrib"], to_torch(G, DEV), bg=bg)
+    for k, v in g.items():
+        a, r = v.cpu().numpy().reshape(b["n"], -1), ref[k].reshape(b["n"], -1)
+        scale = np.abs(r).max(axis=1) + 1e-3 * np.abs(r).max()
+        assert (np.abs(a - r).max(axis=1) / scale).max() <= 2e-4, k
+
+
+@pytest.mark.parametrize("wide", [False, True])
+@pytest.mark.parametrize("early", [False, True])
+def test_fp32_blending_does_not_depend_on_what_is_not_blended(tc, wide, early):
+    """The same fragments with others between them that no pixel blends, half of which pass the block test (a
+    footprint between the pixel centres): batches and groups fall elsewhere, image, transmittance and every
+    gradient stay the same bit for bit.  So do they without the block tests."""
+    rng = np.random.default_rng(7 + wide)
+    cam, inp, b = _pair_case(rng, LENGTHS, wide)
+    n, m = b["n"], 300
+    tile = rng.integers(1, 9, m)
+    pad = dict(mean2d=f32(np.stack([tile % 3 * 16 + rng.integers(1, 16, m), tile // 3 * 16 + rng.integers(1, 16, m)], 1)),
+               conic=f32(np.tile([3.3, 0.0, 3.3], (m, 1))), opacity=f32(np.where(np.arange(m) % 2, 0.005, 0.002)),
+               rgb=f32(rng.uniform(0, 1, (m, 3))))
+    both = {k: np.concatenate([inp[k], pad[k]]) for k in inp}
+    ids, ranges = [], np.zeros((9, 2), np.int64)
+    for t in range(9):
+        own = list(range(*b["ranges"][t]))
+        for k in n + np.nonzero(tile == t)[0]:
+            own.insert(int(rng.integers(0, len(own) + 1)), int(k))
+        ranges[t] = len(ids), len(ids) + len(own)
+        ids += own
+    bp = dict(ids=np.array(ids), ranges=ranges, n=n + m)
+    G = to_torch(f32(rng.standard_normal((3, 40, 40))), DEV)
+    res = []
+    for c, lists_of, cull in ((inp, b, True), (inp, b, False), (both, bp, True)):
+        d, lists, f = _render(tc, cam, c, lists_of, early_cull=early, tile_cull=cull)
+        g = tc.tcgs_render_bwd(cam, tc.render_opts("fp32", early_cull=early), *lists, d["mean2d"], d["conic"], d["opacity"],
+                               d["rgb"], f["img"], f["T_final"], f["n_contrib"], G)
+        res.append((f, g))
+    (f0, g0), (f1, _), (f2, g2) = res
+    for k in ("img", "T_final", "n_contrib"):
+        assert torch.equal(f0[k], f1[k]), k
+    for k in ("img", "T_final"):
+        assert torch.equal(f0[k], f2[k]), k
+    for k in g0:
+        assert torch.equal(g0[k], g2[k][:n]), k
+        assert (g2[k][n:] == 0).all()
+
+
+def test_fp32_blending_keeps_infinities_where_they_are(tc):
+    """An infinite colour or a NaN in dL/dimg reaches only the pixels that blend it and the Gaussians that the
+    pixel blends; conics that are not positive definite or hold a NaN are evaluated at every pixel."""
+    rng = np.random.default_rng(9)
+    cam, inp, b = _pair_case(rng, np.full(9, 40), False)
+    d, lists, clean = _render(tc, cam, inp, b)
+    odd = {k: v.copy() for k, v in inp.items()}
+    odd["rgb"][b["ranges"][4, 0] + 7] = np.inf
+    _, _, f = _render(tc, cam, odd, b)
+    finite = torch.isfinite(f["img"])
+    assert not finite.all() and torch.equal(f["img"][finite], clean["img"][finite])
+    assert torch.equal(f["T_final"], clean["T_final"])
+    for bad in ((np.nan, 0.1, 0.2), (0.01, 0.5, 0.01), (-0.01, 0.0, 0.02)):
+        odd = {k: v.copy() for k, v in inp.items()}
+        odd["conic"][b["ranges"][4, 0] + 7] = f32(bad)
+        _, _, f = _render(tc, cam, odd, b)
+        _, _, every = _render(tc, cam, odd, b, tile_cull=False)
+        for k in ("img", "T_final", "n_contrib"):
+            assert torch.equal(f[k], every[k]), (bad, k)
+
+    G = to_torch(f32(rng.standard_normal((3, 40, 40))), DEV)
+    run = lambda dl: tc.tcgs_render_bwd(cam, tc.render_opts("fp32"), *lists, d["mean2d"], d["conic"], d["opacity"],  # noqa: E731
+                                        d["rgb"], clean["img"], clean["T_final"], clean["n_contrib"], dl)
+    G[:, 20, 20] = 0
+    ref = run(G)
+    lit = torch.zeros_like(G)
+    lit[:, 20, 20] = 1
+    blends = (run(lit)["drgb"] != 0).any(dim=1)
+    G[:, 20, 20] = float("nan")
+    got = run(G)
+    assert blends.any() and not blends.all()
+    for k in ref:
+        assert torch.equal(got[k][~blends], ref[k][~blends]), k
+        assert torch.isnan(got[k][blends]).any()
