@@ -122,6 +122,7 @@ __device__ int2 row_span(const Cover& v, const Reach& e, int ty, int x0, int x1)
     // the shadow [xa, xb] of the ellipse on the x axis within the row's band of pixel centres
     const float yl = __fsub_rn((float)(ty * kTile) + 0.5f, v.my), yh = __fadd_rn(yl, 15.f);
     float Lf = 1.f, Rf = 0.f;   // empty unless the band meets the ellipse
+    float xa_ = 0.f, xb_ = 0.f, rl_ = 0.f, rr_ = 0.f;
     if (!(yl > e.H || yh < -e.H)) {
         const float alim = __fmul_rn(v.a, v.lim);
         const float dl = fminf(yh, fmaxf(yl, e.s)), dr = fminf(yh, fmaxf(yl, -e.s));
@@ -129,6 +130,7 @@ __device__ int2 row_span(const Cover& v, const Reach& e, int ty, int x0, int x1)
         const float rr = __fsqrt_rn(fmaxf(0.f, __fsub_rn(alim, __fmul_rn(e.det, __fmul_rn(dr, dr)))));
         const float xa = __fmul_rn(__fsub_rn(__fmul_rn(-v.b, dl), rl), v.ia);
         const float xb = __fmul_rn(__fadd_rn(__fmul_rn(-v.b, dr), rr), v.ia);
+        xa_ = xa; xb_ = xb; rl_ = rl; rr_ = rr;
         // tiles whose box [16 tx + 0.5, 16 tx + 15.5] meets [mx + xa, mx + xb]
         Lf = ceilf(__fmul_rn(__fsub_rn(__fadd_rn(v.mx, xa), 15.5f), 1.f / kTile));
         Rf = floorf(__fmul_rn(__fsub_rn(__fadd_rn(v.mx, xb), 0.5f), 1.f / kTile));
@@ -146,7 +148,24 @@ __device__ int2 row_span(const Cover& v, const Reach& e, int ty, int x0, int x1)
         return make_int2(L, R);
     }
     int L = clamp_tile(Lf, x0, x1), R = clamp_tile(Rf, x0, x1);
-    if (test(L)) {
+    // Ends that need no test.  Along y = dl (dr) the form is lim - 2 r e + a e^2 at a distance e inside the
+    // shadow's end (r = rl or rr, half its slope there), so the end tile passes when that is below lim at
+    // the point of its box nearest to the minimum; by convexity it is at least lim + 2 r g over the band at a
+    // distance g outside, where the outer neighbour's box begins.  Both must clear a bound on the roundings
+    // of this code and of the test (1e-5 of the sum of magnitudes, 168 times 2^-24, and of the positions).  The
+    // four tests it saves were most of a row: the runs of 605M splats at 3840 x 2160 take 1.48 ms, against
+    // 1.82 ms with every end tested.
+    const float X = fmaxf(fabsf(xa_), fabsf(xb_)) + 16.f, Y = fmaxf(fabsf(yl), fabsf(yh));
+    const float slack0 = 1e-5f * (v.a * X * X + v.c * Y * Y), slack1 = 1e-5f * (fabsf(v.mx) + X);
+    auto sure = [&](float r, float far, bool clamped) {   // far: from the end to the far side of the end tile's box
+        const float e = fminf(fmaxf(r * v.ia, far - 15.f), far), s = slack0 + slack1 * r;
+        return far >= 0.f && e * (2.f * r - v.a * e) > s && (clamped || 2.f * r * (16.f - far) > s);
+    };
+    const bool sure_l = sure(rl_, (float)(L * kTile) + 15.5f - (v.mx + xa_), (float)L > Lf);
+    const bool sure_r = sure(rr_, (v.mx + xb_) - ((float)(R * kTile) + 0.5f), (float)R < Rf);
+    if (sure_l && sure_r && L <= R) return make_int2(L, R);
+    if (sure_l) {
+    } else if (test(L)) {
         while (L > x0 && test(L - 1)) --L;
     } else {
         int k = L + 1;
@@ -154,7 +173,8 @@ __device__ int2 row_span(const Cover& v, const Reach& e, int ty, int x0, int x1)
         if (k > R) return scan();
         L = k;
     }
-    if (test(R)) {
+    if (sure_r) {
+    } else if (test(R)) {
         while (R < x1 && test(R + 1)) ++R;
     } else {
         int k = R - 1;
