@@ -31,7 +31,7 @@ constexpr int kChunk = 512;                  // runs expanded together: 16 words
 constexpr int kChunkWords = kChunk / 32;
 constexpr int kSpanBuffer = 3072;            // runs of a span block kept in shared memory (more: evaluated twice)
 constexpr int kScatterStage = 4096;          // runs regrouped by row at a time
-constexpr int kExpandStage = 4096;           // ids regrouped by column at a time
+constexpr int kExpandStage = 3584;           // ids regrouped by column at a time (4 expand blocks an SM up to 256 columns)
 static_assert(kRowThreads == kRowListsMaxGrid && kChunk <= kExpandStage && kRowThreads <= kScatterStage,
               "a thread per row or column; a column of a chunk, or a row of a block, fits the stage");
 
@@ -467,20 +467,25 @@ __global__ void __launch_bounds__(kRowThreads) k_col_counts(int grid_w, int grid
 }
 
 // 5. Block (row, 32 columns): the exclusive prefix of the columns' counts over the row's chunks (in
-// place; each warp sums, then rewrites, one eighth of the chunks), the tiles' lengths and the row's.
-__global__ void __launch_bounds__(kRowThreads) k_col_offsets(int grid_w, RowScratch w) {
+// place; each warp sums, then rewrites, its part of the chunks), the tiles' lengths and the row's.  Bound by
+// the latency of a warp's walk down its chunks in the longest row, hence 32 warps (605M splats at 3840 x 2160:
+// 498 us with 8 warps, 293 us).
+constexpr int kColThreads = 1024;
+constexpr int kColWarps = kColThreads / 32;
+
+__global__ void __launch_bounds__(kColThreads) k_col_offsets(int grid_w, RowScratch w) {
     pdl_trigger();
     pdl_wait();
-    __shared__ uint32_t s_sum[kRowWarps][32];
-    __shared__ uint32_t s_ws[kRowWarps];
+    __shared__ uint32_t s_sum[kColWarps][32];
+    __shared__ uint32_t s_ws[kColWarps];
     if (w.ctr->n_ok == 0u) return;
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     const uint32_t row = blockIdx.x, col = blockIdx.y * 32u + lane;
     const uint32_t r = (uint32_t)t < row ? w.ctr->row_runs[t] : 0u;
     uint32_t chunk0;
-    block_exclusive_scan<uint32_t, kRowThreads>(r / kChunk + (r % kChunk != 0u), s_ws, chunk0);
+    block_exclusive_scan<uint32_t, kColThreads>(r / kChunk + (r % kChunk != 0u), s_ws, chunk0);
     const uint32_t n = w.ctr->row_runs[row], chunks = n / kChunk + (n % kChunk != 0u);
-    const uint32_t per = (chunks + kRowWarps - 1) / kRowWarps;
+    const uint32_t per = (chunks + kColWarps - 1) / kColWarps;
     const uint32_t lo = min((uint32_t)warp * per, chunks), hi = min(lo + per, chunks);
     const bool in = col < (uint32_t)grid_w;
     uint32_t* m = w.m2 + (size_t)chunk0 * grid_w + (in ? col : 0u);
@@ -493,7 +498,7 @@ __global__ void __launch_bounds__(kRowThreads) k_col_offsets(int grid_w, RowScra
     __syncthreads();
     uint32_t run = 0, total = 0;
 #pragma unroll
-    for (int k = 0; k < kRowWarps; ++k) {
+    for (int k = 0; k < kColWarps; ++k) {
         run += k < warp ? s_sum[k][lane] : 0u;
         total += s_sum[k][lane];
     }
@@ -518,19 +523,27 @@ __global__ void __launch_bounds__(kRowThreads) k_col_offsets(int grid_w, RowScra
 // run k covers it; a run's place in column x's part of the chunk is the number of set bits below its
 // own.  The ids are regrouped by column in shared memory (column windows of at most kExpandStage ids)
 // and written out in that order, so that each list's part is one contiguous write.
+// Bound by latency (barriers, shared-memory round trips, the loads of a chunk) at 24 warps an SM, so
+// shared memory is sized by the columns there are (4 blocks an SM, 5 up to 185 columns, instead of 3) and
+// the next chunk's runs are loaded while the current one is regrouped (2.3M splats at 1920 x 1080: 37 -> 26 us,
+// 605M at 3840 x 2160: 2.73 -> 2.46 ms).  A run's columns dealt to several lanes, and the sets formed by a
+// prefix XOR of two toggles a run instead of one atomic a column, both measured slower.
 struct ExpandSmem {
     RowTable tab;
     uint32_t row_base[kRowListsMaxGrid + 1];        // first splat of each row
-    uint32_t bits[kChunkWords * kRowListsMaxGrid];  // [word][column]
-    uint32_t before[kChunkWords * kRowListsMaxGrid];   // place of the word's first run in the chunk's ids
     uint32_t start[kRowListsMaxGrid + 1];           // first id of each column among the chunk's
     uint32_t delta[kRowListsMaxGrid];               // global position minus that
     uint32_t stage[kExpandStage];
     uint8_t stage_col[kExpandStage];
     uint32_t ws[kRowWarps];
+    // then, each [word][column]: the sets' bits, and the place of the word's first run in the chunk's ids
 };
 
-__global__ void __launch_bounds__(kRowThreads) k_row_expand(int grid_w, int grid_h, uint32_t* __restrict__ ids_sorted,
+constexpr int kExpandBlocks = 5;
+
+inline size_t expand_smem_bytes(int grid_w) { return sizeof(ExpandSmem) + 2 * 4 * (size_t)kChunkWords * grid_w; }
+
+__global__ void __launch_bounds__(kRowThreads, kExpandBlocks) k_row_expand(int grid_w, int grid_h, uint32_t* __restrict__ ids_sorted,
                                                             uint32_t* __restrict__ ranges, RowScratch w) {
     pdl_trigger();
     pdl_wait();
@@ -544,11 +557,37 @@ __global__ void __launch_bounds__(kRowThreads) k_row_expand(int grid_w, int grid
     __syncthreads();
     const uint32_t chunks = s.tab.chunk[kRowListsMaxGrid];
     const uint32_t below = (1u << (t & 31)) - 1u;
+    uint32_t* const bits = reinterpret_cast<uint32_t*>(smem + sizeof(ExpandSmem));
+    uint32_t* const before = bits + kChunkWords * grid_w;
     uint32_t at_row = 0xFFFFFFFFu, list = 0;   // list: first splat of column t of the row
-    for (uint32_t c = blockIdx.x; c < chunks; c += gridDim.x) {
+    constexpr int kEach = kChunk / kRowThreads;
+    uint32_t next_row, next_id[kEach], next_sp[kEach];   // the next chunk's runs of this thread; an empty span: none
+    auto fetch = [&](uint32_t c) {
         uint32_t first, n;
-        const uint32_t row = chunk_row(s.tab, c, first, n);
-        for (int k = t; k < kChunkWords * grid_w; k += kRowThreads) s.bits[k] = 0u;
+        next_row = chunk_row(s.tab, c, first, n);
+#pragma unroll
+        for (int q = 0; q < kEach; ++q) {
+            const uint32_t k = (uint32_t)(q * kRowThreads + t);
+            next_id[q] = 0u;
+            next_sp[q] = 1u;   // first 1, last 0
+            if (k < n) {
+                next_sp[q] = w.run_span[first + k];
+                next_id[q] = w.run_id[first + k];
+            }
+        }
+    };
+    if (blockIdx.x < chunks) fetch(blockIdx.x);
+    for (uint32_t c = blockIdx.x; c < chunks; c += gridDim.x) {
+        const uint32_t row = next_row;
+        uint32_t id[kEach], x0[kEach], x1[kEach];
+#pragma unroll
+        for (int q = 0; q < kEach; ++q) {
+            id[q] = next_id[q];
+            x0[q] = next_sp[q] & 0xFFu;
+            x1[q] = next_sp[q] >> 8;
+        }
+        const uint32_t in_tile = t < grid_w ? w.m2[(size_t)c * grid_w + t] : 0u;
+        for (int k = t; k < kChunkWords * grid_w; k += kRowThreads) bits[k] = 0u;
         if (row != at_row) {
             const uint32_t len = t < grid_w ? w.tile_count[row * (uint32_t)grid_w + t] : 0u;
             list = s.row_base[row] + block_exclusive_scan<uint32_t, kRowThreads>(len, s.ws, tot);
@@ -559,37 +598,28 @@ __global__ void __launch_bounds__(kRowThreads) k_row_expand(int grid_w, int grid
             }
         }
         __syncthreads();
-        uint32_t id[kChunk / kRowThreads], x0[kChunk / kRowThreads], x1[kChunk / kRowThreads];
 #pragma unroll
-        for (int q = 0; q < kChunk / kRowThreads; ++q) {
-            const uint32_t k = (uint32_t)(q * kRowThreads + t);
-            id[q] = 0u;
-            x0[q] = 1u; x1[q] = 0u;
-            if (k < n) {
-                const uint32_t sp = w.run_span[first + k];
-                id[q] = w.run_id[first + k];
-                x0[q] = sp & 0xFFu;
-                x1[q] = sp >> 8;
-                for (uint32_t x = x0[q]; x <= x1[q]; ++x)
-                    atomicOr(&s.bits[(k >> 5) * (uint32_t)grid_w + x], 1u << (t & 31));
-            }
+        for (int q = 0; q < kEach; ++q) {
+            uint32_t* word = bits + (uint32_t)((q * kRowThreads + t) >> 5) * (uint32_t)grid_w;
+            for (uint32_t x = x0[q]; x <= x1[q]; ++x) atomicOr(&word[x], 1u << (t & 31));
         }
+        if (c + gridDim.x < chunks) fetch(c + gridDim.x);
         __syncthreads();
         uint32_t len = 0;
         if (t < grid_w) {
 #pragma unroll
-            for (int g = 0; g < kChunkWords; ++g) len += __popc(s.bits[g * grid_w + t]);
+            for (int g = 0; g < kChunkWords; ++g) len += __popc(bits[g * grid_w + t]);
         }
         const uint32_t start = block_exclusive_scan<uint32_t, kRowThreads>(len, s.ws, tot);
         s.start[t] = start;
         if (t == 0) s.start[kRowListsMaxGrid] = tot;
         if (t < grid_w) {
-            s.delta[t] = list + w.m2[(size_t)c * grid_w + t] - start;
+            s.delta[t] = list + in_tile - start;
             uint32_t run = start;
 #pragma unroll
             for (int g = 0; g < kChunkWords; ++g) {
-                s.before[g * grid_w + t] = run;
-                run += __popc(s.bits[g * grid_w + t]);
+                before[g * grid_w + t] = run;
+                run += __popc(bits[g * grid_w + t]);
             }
         }
         __syncthreads();
@@ -597,13 +627,13 @@ __global__ void __launch_bounds__(kRowThreads) k_row_expand(int grid_w, int grid
             const uint32_t c1 = window_end(s.start, c0, (uint32_t)grid_w, kExpandStage);
             const uint32_t base = s.start[c0], items = s.start[c1] - base;
 #pragma unroll
-            for (int q = 0; q < kChunk / kRowThreads; ++q) {
+            for (int q = 0; q < kEach; ++q) {
                 const uint32_t at = (uint32_t)(q * kRowThreads + t) >> 5;
                 const uint32_t lo = x0[q] > c0 ? x0[q] : c0, hi = x1[q] < c1 - 1 ? x1[q] : c1 - 1;
                 if (x0[q] <= x1[q])
                     for (uint32_t x = lo; x <= hi; ++x) {
                         const uint32_t k = at * (uint32_t)grid_w + x;
-                        const uint32_t p = s.before[k] - base + __popc(s.bits[k] & below);
+                        const uint32_t p = before[k] - base + __popc(bits[k] & below);
                         s.stage[p] = id[q];
                         s.stage_col[p] = (uint8_t)x;
                     }
@@ -617,15 +647,16 @@ __global__ void __launch_bounds__(kRowThreads) k_row_expand(int grid_w, int grid
     }
 }
 
-// Blocks of a persistent kernel resident at once on the current device (looked up once per device).
+// Blocks of a persistent kernel resident at once on the current device, looked up once per device (and
+// number of columns, on which the expansion's shared memory depends).
 template <typename K>
-int resident_blocks(K kern, int threads, size_t smem, int (&cached)[kMaxDevices]) {
+int resident_blocks(K kern, int threads, size_t smem, size_t max_smem, int (&cached)[kMaxDevices]) {
     static std::mutex mu;
     DeviceInfo d;
     if (!current_device_info(&d)) return 256;
     std::lock_guard<std::mutex> lock(mu);
     if (cached[d.device] == 0) {
-        if (smem) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (max_smem) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_smem);
         int per_sm = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
         cached[d.device] = d.sms * (per_sm > 0 ? per_sm : 1);
@@ -662,13 +693,14 @@ void launch_row_lists(const RowLists& a, cudaStream_t s) {
     if (a.capacity == 0) return;   // N and the status are settled; there is nothing to place
     launch_pdl(k_row_scatter, nb, kRowThreads, 0, s, a.P, a.order, gh, nb, w);
     // at most capacity / kChunk + grid_h chunks
-    static int count_blocks[kMaxDevices] = {}, expand_blocks[kMaxDevices] = {};
+    static int count_blocks[kMaxDevices] = {}, expand_blocks[kRowListsMaxGrid + 1][kMaxDevices] = {};
+    const size_t smem = expand_smem_bytes(gw);
     const int64_t chunks = a.capacity / kChunk + gh;
-    const int64_t cb = resident_blocks(k_col_counts, kRowThreads, 0, count_blocks);
-    const int64_t eb = resident_blocks(k_row_expand, kRowThreads, sizeof(ExpandSmem), expand_blocks);
+    const int64_t cb = resident_blocks(k_col_counts, kRowThreads, 0, 0, count_blocks);
+    const int64_t eb = resident_blocks(k_row_expand, kRowThreads, smem, expand_smem_bytes(kRowListsMaxGrid), expand_blocks[gw]);
     launch_pdl(k_col_counts, (int)(chunks < cb ? chunks : cb), kRowThreads, 0, s, gw, gh, w);
-    launch_pdl(k_col_offsets, dim3(gh, (gw + 31) / 32), kRowThreads, 0, s, gw, w);
-    launch_pdl(k_row_expand, (int)(chunks < eb ? chunks : eb), kRowThreads, sizeof(ExpandSmem), s, gw, gh, a.ids_sorted,
+    launch_pdl(k_col_offsets, dim3(gh, (gw + 31) / 32), kColThreads, 0, s, gw, w);
+    launch_pdl(k_row_expand, (int)(chunks < eb ? chunks : eb), kRowThreads, smem, s, gw, gh, a.ids_sorted,
                a.ranges, w);
     count_launches(4);
 }
