@@ -232,3 +232,76 @@ def test_fp32_blending_keeps_infinities_where_they_are(tc):
     for k in ref:
         assert torch.equal(got[k][~blends], ref[k][~blends]), k
         assert torch.isnan(got[k][blends]).any()
+
+
+@pytest.mark.parametrize("P", [1, 31, 32, 33, 1023, 1025, 3000])
+def test_small_view_depth_order_edges(tc, P):
+    """Counts around the ranking kernel's 32 Gaussians a block and 1024 keys a tile, with depth ties and culled
+    Gaussians: the oracle's lists; N and the status when the capacity is N and N - 1."""
+    cam = scenes.pinhole(100, 70, fx=100.0)
+    rng = np.random.default_rng(P)
+    mean2d = f32(rng.uniform(-10, 110, (P, 2)))
+    radius = rng.integers(0, 12, P).astype(np.int32)
+    depth = f32(rng.integers(1, max(2, P // 3), P))
+    b = oracle.bin_sort(cam, mean2d, radius, depth)
+    d = [to_torch(v, DEV) for v in (mean2d, radius, depth)]
+    for cap in (b["n"], max(b["n"] - 1, 0)):
+        assert cap <= 32768
+        o = tc.tcgs_bin_sort(cam, *d, cap)
+        assert int(o["n_splats"].item()) == b["n"]
+        if cap == b["n"]:
+            assert int(o["status"].item()) == 0
+            assert (o["ids_sorted"].cpu().numpy()[:cap] == b["ids"]).all()
+            got, ref = o["tile_ranges"].cpu().numpy(), b["ranges"]
+            assert ((got == ref) | (ref[:, :1] == ref[:, 1:]) & (got[:, :1] == got[:, 1:])).all()
+        else:
+            assert int(o["status"].item()) == 3
+
+
+def _tile_lists(o, gw, cols):
+    """Lengths [rows, cols] and the concatenated ids of the lists of the first `cols` columns."""
+    r = o["tile_ranges"].cpu().numpy().astype(np.int64).reshape(-1, gw, 2)[:, :cols]
+    lens = r[..., 1] - r[..., 0]
+    at = np.repeat(r[..., 0].ravel() - (np.cumsum(lens) - lens.ravel()), lens.ravel()) + np.arange(int(lens.sum()))
+    return lens, o["ids_sorted"].cpu().numpy()[at]
+
+
+@pytest.mark.parametrize("height", [640, 4096])
+@pytest.mark.parametrize("mode", ["rectangles", "tiles", "rows"])
+def test_row_lists_equal_radix_lists(tc, height, mode):
+    """A view of 256 tile columns (sorted by row lists) against the same Gaussians in one of 257 (sorted by
+    radix passes): every list of the common columns is the same.  Narrow and wide footprints, blocks of
+    256 Gaussians with more runs than the kernels keep in shared memory, rows and columns of many chunks, and
+    (exact coverage) conics that are not positive definite or hold a NaN, whose rows are reached in parts."""
+    rng = np.random.default_rng(len(mode) + height)
+    P = 3000
+    wide = np.arange(P) % 3 == 0
+    sigma = np.where(wide, rng.uniform(*((5, 20) if mode == "tiles" else (60, 220)), P), rng.uniform(0.5, 6, P))
+    mean2d = np.stack([rng.uniform(-30, 3500, P), rng.uniform(-30, height + 30, P)], 1)
+    mean2d[1500:2200] = rng.uniform(0, 300, (700, 2))       # long lists in a corner
+    c = 0.9 * rng.uniform(-1, 1, P)
+    conic = np.stack([1 / sigma ** 2, c / sigma ** 2, 1 / sigma ** 2], 1) / (1 - c * c)[:, None]
+    odd = rng.choice(np.nonzero(mean2d[:, 0] < 2500)[0], 60, replace=False)
+    conic[odd[:20], 1] = 2 * conic[odd[:20], 0]             # hyperbolic
+    conic[odd[20:40], 0] *= -1
+    conic[odd[40:]] = np.nan
+    opacity = rng.uniform(0.003, 1, P)
+    radius = np.ceil(3 * sigma).astype(np.int32)
+    radius[rng.choice(P, 100, replace=False)] = 0
+    mean2d, conic, opacity = f32(mean2d), f32(conic), f32(opacity)
+    depth = f32(rng.integers(1, 500, P))
+    d = [to_torch(v, DEV) for v in (mean2d, radius, depth)]
+    exact = dict(conic=to_torch(conic, DEV), opacity=to_torch(opacity, DEV)) if mode != "rectangles" else {}
+    n = int(oracle.bin_sort(scenes.pinhole(4112, height, fx=500.0), mean2d, radius, depth)["n"])
+    # the capacity chooses the coverage by tiles or by rows in both paths
+    cap = max(n, 32 * P) if mode != "tiles" else 32 * P - 1
+    res = [tc.tcgs_bin_sort(scenes.pinhole(16 * gw, height, fx=500.0), *d, cap, **exact) for gw in (256, 257)]
+    assert n <= cap
+    assert int(res[0]["status"].item()) == int(res[1]["status"].item()) == 0
+    (la, ia), (lb, ib) = _tile_lists(res[0], 256, 256), _tile_lists(res[1], 257, 256)
+    assert (la == lb).all() and (ia == ib).all()
+    assert la.sum() == int(res[0]["n_splats"].item())
+    again = tc.tcgs_bin_sort(scenes.pinhole(4096, height, fx=500.0), *d, int(la.sum()) - 1, **exact)
+    assert int(again["status"].item()) == 3
+    if mode == "rectangles":
+        assert int(again["n_splats"].item()) == la.sum()
