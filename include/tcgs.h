@@ -93,7 +93,7 @@ typedef struct {
                                 0 = cull on alpha < 1/255 after it (Eq. 5, the 3DGS baseline).  On the TC paths
                                 the walk is branch-free and evaluates ex2 for every walked fragment either way:
                                 the option changes the test, not the work */
-    int32_t tile_cull;       /* TC paths: 1 = skip, per 8x4 pixel block, list entries whose Gaussian cannot
+    int32_t tile_cull;       /* 1 = skip, per 8x4 pixel block (TCGS_FP32: 8x8), list entries whose Gaussian cannot
                                 reach alpha >= 1/255 at any pixel of the block (exact minimum of the conic
                                 form over the block; the image is unchanged); 0 = walk every entry */
     uint32_t* tile_stats;    /* nullable device [num_tiles * 8], accumulated (+=) per tile:
@@ -109,7 +109,8 @@ typedef struct {
                                 order, a permutation of all tiles such as tcgs_tile_order's (the order
                                 changes the schedule, never the image); NULL: one CTA per tile.  A view
                                 of at most tcgs_tc_wave_tiles() tiles is rendered one CTA per tile even
-                                when an order is given: every tile then starts in the first wave */
+                                when an order is given: every tile then starts in the first wave.
+                                TCGS_FP32 and tcgs_render_bwd start one CTA per tile in this order */
     uint32_t* work_counter;  /* device uint32, required with tile_order: the grid's next-tile counter,
                                 zeroed by the call */
     int32_t pixels_per_thread; /* 0 or 1: the tensor-core renderer's consumer threads blend one pixel
@@ -188,10 +189,12 @@ TCGS_API size_t tcgs_bin_sort_workspace_size(int32_t P, int64_t splat_capacity, 
  * The order is the (tile, depth-bits) key order of the paper's radix sort; it is produced by
  * an LSD radix sort whose depth digits run before duplication (on P keys) and whose tile
  * digits run after it (on N keys).  A small view (at most 256 tiles, P <= 8192 and
- * splat_capacity <= 32768) runs the same passes in two single-CTA kernels (4 launches in all,
- * against about 20), with the same result.  With two tile passes and splat_capacity >= 2^23, the
- * first tile pass packs (tile >> 8, Gaussian id) into one word when they fit 32 bits, and the second
- * writes the ranges from per-tile counts: again the same result.  Empty tiles get [0, 0).
+ * splat_capacity <= 32768) is ranked by counting and sorted by tile in one CTA (4 launches in all,
+ * against about 20), and any other view of at most 256 x 256 tiles is sorted by tile-row lists (runs of
+ * tiles instead of splats), with the same result.  In the radix sort of larger views, with two tile passes
+ * and splat_capacity >= 2^23, the first tile pass packs (tile >> 8, Gaussian id) into one word when they
+ * fit 32 bits, and the second writes the ranges from per-tile counts: again the same result.  Empty tiles
+ * get [0, 0).
  * In:  mean2d [P,2], radius [P], depth [P] (> 0 where radius > 0).
  * Out: ids_sorted [splat_capacity] uint32 (first N entries valid), tile_ranges [num_tiles, 2]
  *      uint32 [start, end), n_splats: device int64 = N, status: device int32 (TCGS_OK, or

@@ -9,6 +9,7 @@ namespace {
 struct FwdParams {
     DevCamera cam;
     const uint32_t* ranges;
+    const uint32_t* order;   // nullable: the tile of each CTA
     const uint32_t* ids;
     const float* mean2d;
     const float* conic;
@@ -59,7 +60,8 @@ __global__ void __launch_bounds__(kFwdThreads, 7) k_render_fp32(FwdParams p) {
     __shared__ __align__(4) uint8_t s_list[kFwdWarps][kFwdBatch + kFwdGroup];
     const long long t_start = kStats ? clock64() : 0;
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-    const int tile = blockIdx.x;
+    const int tile = p.order ? (int)p.order[blockIdx.x] : (int)blockIdx.x;
+    if (tile < 0 || tile >= p.cam.grid_w * p.cam.grid_h) return;   // never index past the grid
     const int tx = tile % p.cam.grid_w, ty = tile / p.cam.grid_w;
     const PairPixels q = pair_pixels(warp, lane);
     const float cx = (float)(tx * kTile + kTile / 2), cy = (float)(ty * kTile + kTile / 2);
@@ -249,6 +251,7 @@ __global__ void __launch_bounds__(kFwdThreads, 7) k_render_fp32(FwdParams p) {
 struct BwdParams {
     DevCamera cam;
     const uint32_t* ranges;
+    const uint32_t* order;   // nullable: the tile of each CTA
     const uint32_t* ids;
     const float* mean2d;
     const float* conic;
@@ -274,14 +277,15 @@ constexpr int kBwdGroup = 4;             // fragments replayed together: one per
 constexpr int kBwdParams = 9;            // dmean2d (2), dconic (3), dopacity, drgb (3), up to constant factors
 
 template <bool kEarly>
-__global__ void __launch_bounds__(kBwdThreads, 5) k_render_bwd(BwdParams p) {
+__global__ void __launch_bounds__(kBwdThreads, 4) k_render_bwd(BwdParams p) {
     __shared__ PairRec s_f[kBwdBatch + 1];                             // the last record contributes nothing
     __shared__ float s_part[kBwdWarps][kBwdBatch + 1][kBwdParams];
     __shared__ uint32_t s_mark[2][kBwdWarps][kBwdBatch / 32];          // per block: fragments to replay
     __shared__ __align__(4) uint8_t s_list[kBwdWarps][kBwdBatch + kBwdGroup];
     __shared__ uint32_t s_max;
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-    const int tile = blockIdx.x;
+    const int tile = p.order ? (int)p.order[blockIdx.x] : (int)blockIdx.x;
+    if (tile < 0 || tile >= p.cam.grid_w * p.cam.grid_h) return;   // never index past the grid
     const int tx = tile % p.cam.grid_w, ty = tile / p.cam.grid_w;
     const PairPixels q = pair_pixels(warp, lane);
     const float cx = (float)(tx * kTile + kTile / 2), cy = (float)(ty * kTile + kTile / 2);
@@ -375,47 +379,47 @@ __global__ void __launch_bounds__(kBwdThreads, 5) k_render_bwd(BwdParams p) {
         __syncwarp();
         for (uint32_t at = 0; at < n; at += kBwdGroup) {
             const uint32_t four = *reinterpret_cast<const uint32_t*>(&s_list[warp][at]);
+            // alphas of the four fragments (negated; 0: the pixel does not blend it), exp(power) (0: or with a
+            // clamped alpha), dx, dy
+            f32x2 na[kBwdGroup], G[kBwdGroup], dx[kBwdGroup], dy[kBwdGroup];
+            bool any = false;
+#pragma unroll
+            for (int f = 0; f < kBwdGroup; ++f) {
+                const uint32_t j = (four >> (8 * f)) & 0xFFu;
+                const PairRec& r = s_f[j];
+                const ulonglong2 xa = r.q[0], bc = r.q[1], yo = r.q[2];
+                dx[f] = add2(xa.x, npx);
+                dy[f] = add2(yo.x, npy);
+                const f32x2 pw = pair_power(xa.y, bc.x, bc.y, dx[f], dy[f]);
+                const float G0 = expf(lo2(pw)), G1 = expf(hi2(pw));
+                const f32x2 raw = mul2(yo.y, pack2f(G0, G1));   // -o exp(power)
+                const float a0 = fmaxf(-amax, lo2(raw)), a1 = fmaxf(-amax, hi2(raw));
+                bool in0 = a0 <= -kCullAlpha && b0 + j < nc[0], in1 = a1 <= -kCullAlpha && b0 + j < nc[1];
+                if (kEarly) {   // the forward's test
+                    const float lno = r.lno();
+                    in0 = in0 && !(lo2(pw) + lno < kBetaCull);
+                    in1 = in1 && !(hi2(pw) + lno < kBetaCull);
+                }
+                any = any || in0 || in1;
+                na[f] = pack2f(in0 ? a0 : 0.f, in1 ? a1 : 0.f);
+                G[f] = pack2f(in0 && lo2(raw) >= -amax ? G0 : 0.f, in1 && hi2(raw) >= -amax ? G1 : 0.f);
+            }
             const bool u16 = lane & 16, u8 = lane & 8, u4 = lane & 4, u2 = lane & 2, u1 = lane & 1;
             const uint32_t jl = (four >> ((u16 ? 8 : 0) + (u8 ? 16 : 0))) & 0xFFu;   // this quarter's fragment
             float* part = s_part[warp][jl];
+            if (!__any_sync(0xffffffffu, any)) {
+                part[lane & 7] = 0.f;
+                part[8] = 0.f;
+                continue;
+            }
             float z[2][kBwdParams];
 #pragma unroll
-            for (int h = 0; h < kBwdGroup; h += 2) {
-                // alphas of two fragments (negated; 0: the pixel does not blend it), exp(power) (0: or with a
-                // clamped alpha), dx, dy
-                f32x2 na[2], G[2], dx[2], dy[2];
-                bool any = false;
-#pragma unroll
-                for (int f = 0; f < 2; ++f) {
-                    const uint32_t j = (four >> (8 * (h + f))) & 0xFFu;
-                    const PairRec& r = s_f[j];
-                    const ulonglong2 xa = r.q[0], bc = r.q[1], yo = r.q[2];
-                    dx[f] = add2(xa.x, npx);
-                    dy[f] = add2(yo.x, npy);
-                    const f32x2 pw = pair_power(xa.y, bc.x, bc.y, dx[f], dy[f]);
-                    const float G0 = expf(lo2(pw)), G1 = expf(hi2(pw));
-                    const f32x2 raw = mul2(yo.y, pack2f(G0, G1));   // -o exp(power)
-                    const float a0 = fmaxf(-amax, lo2(raw)), a1 = fmaxf(-amax, hi2(raw));
-                    bool in0 = a0 <= -kCullAlpha && b0 + j < nc[0], in1 = a1 <= -kCullAlpha && b0 + j < nc[1];
-                    if (kEarly) {   // the forward's test
-                        const float lno = r.lno();
-                        in0 = in0 && !(lo2(pw) + lno < kBetaCull);
-                        in1 = in1 && !(hi2(pw) + lno < kBetaCull);
-                    }
-                    any = any || in0 || in1;
-                    na[f] = pack2f(in0 ? a0 : 0.f, in1 ? a1 : 0.f);
-                    G[f] = pack2f(in0 && lo2(raw) >= -amax ? G0 : 0.f, in1 && hi2(raw) >= -amax ? G1 : 0.f);
-                }
-                if (!__any_sync(0xffffffffu, any)) {   // a warp's pixels may have ended, or lie between the centres
-#pragma unroll
-                    for (int k = 0; k < kBwdParams; ++k) z[h / 2][k] = 0.f;
-                    continue;
-                }
+            for (int f = 0; f < kBwdGroup; f += 2) {
                 float v[2][kBwdParams];
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
-                    const f32x2 na_f = na[e], G_f = G[e], dx_f = dx[e], dy_f = dy[e];
-                    const PairRec& r = s_f[(four >> (8 * (h + e))) & 0xFFu];
+                    const f32x2 na_f = na[f + e], G_f = G[f + e], dx_f = dx[f + e], dy_f = dy[f + e];
+                    const PairRec& r = s_f[(four >> (8 * (f + e))) & 0xFFu];
                     f32x2 cr = r.q[3].x, cg = r.q[3].y, cb = r.q[4].x, h0 = ng0, h1 = ng1, h2 = ng2;
                     if (strict) {   // 0 times an infinity or a NaN would reach what does not blend it
                         cr = where2(na_f, cr); cg = where2(na_f, cg); cb = where2(na_f, cb);
@@ -457,7 +461,7 @@ __global__ void __launch_bounds__(kBwdThreads, 5) k_render_bwd(BwdParams p) {
                     T = fma2(na_f, T, T);
                 }
 #pragma unroll
-                for (int k = 0; k < kBwdParams; ++k) z[h / 2][k] = exchange(v[0][k], v[1][k], u16, 16);
+                for (int k = 0; k < kBwdParams; ++k) z[f / 2][k] = exchange(v[0][k], v[1][k], u16, 16);
             }
             float y[kBwdParams];
 #pragma unroll
@@ -507,7 +511,7 @@ tcgs_status launch_render_fp32(const tcgs_camera* cam, const tcgs_render_opts* o
                                uint32_t* n_contrib, cudaStream_t s) {
     FwdParams p;
     p.cam = make_dev_camera(*cam);
-    p.ranges = tile_ranges; p.ids = ids_sorted; p.mean2d = mean2d; p.conic = conic; p.opacity = opacity;
+    p.ranges = tile_ranges; p.order = opts->tile_order; p.ids = ids_sorted; p.mean2d = mean2d; p.conic = conic; p.opacity = opacity;
     p.rgb = rgb;
     for (int i = 0; i < 3; ++i) p.bg[i] = bg3 ? bg3[i] : 0.f;
     p.alpha_max = opts->alpha_max;
@@ -543,7 +547,7 @@ extern "C" tcgs_status tcgs_render_bwd(const tcgs_camera* cam, const tcgs_render
     if (reinterpret_cast<uintptr_t>(mean2d) & 7) return TCGS_ERR_INVALID;
     BwdParams p;
     p.cam = make_dev_camera(*cam);
-    p.ranges = tile_ranges; p.ids = ids_sorted; p.mean2d = mean2d; p.conic = conic; p.opacity = opacity;
+    p.ranges = tile_ranges; p.order = opts->tile_order; p.ids = ids_sorted; p.mean2d = mean2d; p.conic = conic; p.opacity = opacity;
     p.rgb = rgb;
     for (int i = 0; i < 3; ++i) p.bg[i] = bg3 ? bg3[i] : 0.f;
     p.alpha_max = opts->alpha_max;
