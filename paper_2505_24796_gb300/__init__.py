@@ -38,13 +38,15 @@ def _L():
 
 def _stream(stream=None) -> int:
     if stream is None:
-        return torch.cuda.current_stream().cuda_stream
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 def _ptr(t: torch.Tensor | None, dtype=None, name="tensor") -> int | None:
     if t is None:
         return None
+    if t.is_cuda and t.is_contiguous() and (dtype is None or t.dtype is dtype):
+        return t.data_ptr()
     if not t.is_cuda:
         raise ValueError(f"{name} must be a CUDA tensor (no CPU path exists)")
     if not t.is_contiguous():
@@ -52,6 +54,13 @@ def _ptr(t: torch.Tensor | None, dtype=None, name="tensor") -> int | None:
     if dtype is not None and t.dtype != dtype:
         raise ValueError(f"{name} must be {dtype}, got {t.dtype}")
     return t.data_ptr()
+
+
+def _zeros(*like) -> list:
+    """Zeroed tensors of the given (shape, device): one fill for all of them."""
+    out = [torch.empty(shape, device=dev) for shape, dev in like]
+    torch._foreach_zero_(out)
+    return out
 
 
 def make_camera(cam: dict) -> tcgs_camera:
@@ -123,8 +132,8 @@ def tcgs_project_bwd(cam, means3, scales, quats, sh, sh_degree, radius, dmean2d,
     c = _cam(cam)
     P = means3.shape[0]
     if grads is None:
-        grads = dict(dmeans3=torch.zeros_like(means3), dscales=torch.zeros_like(scales),
-                     dquats=torch.zeros_like(quats), dsh=torch.zeros_like(sh))
+        grads = dict(zip(("dmeans3", "dscales", "dquats", "dsh"),
+                         _zeros(*((t.shape, t.device) for t in (means3, scales, quats, sh)))))
     f = torch.float32
     check("tcgs_project_bwd", _L().tcgs_project_bwd(
         ctypes.byref(c), P, int(sh_degree), _ptr(means3, f, "means3"), _ptr(scales, f, "scales"),
@@ -256,8 +265,8 @@ def tcgs_render_bwd(cam, opts, tile_ranges, ids_sorted, mean2d, conic, opacity, 
     P = mean2d.shape[0]
     dev = mean2d.device
     if grads is None:
-        grads = dict(dmean2d=torch.zeros(P, 2, device=dev), dconic=torch.zeros(P, 3, device=dev),
-                     dopacity=torch.zeros(P, device=dev), drgb=torch.zeros(P, 3, device=dev))
+        grads = dict(zip(("dmean2d", "dconic", "dopacity", "drgb"),
+                         _zeros(((P, 2), dev), ((P, 3), dev), ((P,), dev), ((P, 3), dev))))
     bg3 = (ctypes.c_float * 3)(*[float(b) for b in bg])
     f = torch.float32
     check("tcgs_render_bwd", _L().tcgs_render_bwd(
@@ -585,22 +594,31 @@ class FramePipeline:
 
 # ---------------------------------------------------------------- autograd
 
+def _training_order(cam, tile_ranges):
+    """Longest-first tile order and the renderer's counter for views of more tiles than one wave (else None):
+    the forward and the backward then start their longest tiles first instead of ending with them."""
+    if tile_ranges.shape[0] <= tcgs_tc_wave_tiles():
+        return None, None
+    return (tcgs_tile_order(cam, tile_ranges), torch.empty(1, dtype=torch.int32, device=tile_ranges.device))
+
+
 class _Rasterize(torch.autograd.Function):
     @staticmethod
     def forward(ctx, mean2d, conic, opacity, rgb, cam, tile_ranges, ids_sorted, precision, alpha_max, bg):
-        out = tcgs_render_fwd(cam, render_opts(precision, alpha_max), tile_ranges, ids_sorted, mean2d, conic,
-                              opacity, rgb, bg=bg)
+        order, counter = _training_order(cam, tile_ranges)
+        out = tcgs_render_fwd(cam, render_opts(precision, alpha_max, tile_order=order, work_counter=counter),
+                              tile_ranges, ids_sorted, mean2d, conic, opacity, rgb, bg=bg)
         ctx.cam, ctx.alpha_max, ctx.bg = cam, alpha_max, bg
         ctx.save_for_backward(mean2d, conic, opacity, rgb, tile_ranges, ids_sorted, out["img"], out["T_final"],
-                              out["n_contrib"])
+                              out["n_contrib"], order)
         ctx.mark_non_differentiable(out["T_final"])
         return out["img"], out["T_final"]
 
     @staticmethod
     def backward(ctx, g_img, g_T):
-        mean2d, conic, opacity, rgb, ranges, ids, img, T_final, n_contrib = ctx.saved_tensors
-        g = tcgs_render_bwd(ctx.cam, render_opts("fp32", ctx.alpha_max), ranges, ids, mean2d, conic, opacity, rgb,
-                            img, T_final, n_contrib, g_img.contiguous(), bg=ctx.bg)
+        mean2d, conic, opacity, rgb, ranges, ids, img, T_final, n_contrib, order = ctx.saved_tensors
+        g = tcgs_render_bwd(ctx.cam, render_opts("fp32", ctx.alpha_max, tile_order=order), ranges, ids, mean2d, conic,
+                            opacity, rgb, img, T_final, n_contrib, g_img.contiguous(), bg=ctx.bg)
         return g["dmean2d"], g["dconic"], g["dopacity"], g["drgb"], None, None, None, None, None, None
 
 
@@ -612,25 +630,45 @@ def rasterize(mean2d, conic, opacity, rgb, cam, tile_ranges, ids_sorted, precisi
                             tuple(bg))
 
 
-class _Project(torch.autograd.Function):
-    @staticmethod
-    def forward(ctx, means3, scales, quats, sh, cam, sh_degree, radius_opacity):
-        out = tcgs_project(cam, means3, scales, quats, sh, sh_degree, opacity=radius_opacity)
-        ctx.cam, ctx.sh_degree = cam, sh_degree
-        ctx.save_for_backward(means3, scales, quats, sh, out["radius"])
-        ctx.mark_non_differentiable(out["depth"], out["radius"], out["tiles_touched"])
-        return out["mean2d"], out["conic"], out["rgb"], out["depth"], out["radius"], out["tiles_touched"]
+class _RenderGaussians(torch.autograd.Function):
+    """project -> bin_sort -> render as one node: its backward is tcgs_render_bwd, then tcgs_project_bwd."""
 
     @staticmethod
-    def backward(ctx, g_mean2d, g_conic, g_rgb, g_depth, g_radius, g_tiles):
-        means3, scales, quats, sh, radius = ctx.saved_tensors
-        zeros = lambda t, g: g.contiguous() if g is not None else torch.zeros_like(t)
-        P = means3.shape[0]
-        dev = means3.device
-        g = tcgs_project_bwd(ctx.cam, means3, scales, quats, sh, ctx.sh_degree, radius,
-                             zeros(torch.empty(P, 2, device=dev), g_mean2d), zeros(torch.empty(P, 3, device=dev), g_conic),
-                             zeros(torch.empty(P, 3, device=dev), g_rgb))
-        return g["dmeans3"], g["dscales"], g["dquats"], g["dsh"], None, None, None
+    def forward(ctx, means3, scales, quats, opacity, sh, cam, sh_degree, precision, alpha_max, bg, tight_radius,
+                capacity, exact_tiles):
+        pr = tcgs_project(cam, means3, scales, quats, sh, sh_degree, opacity=opacity if tight_radius else None)
+        if capacity is None:
+            capacity = int(pr["tiles_touched"].sum().item()) + 1   # the sum of int32 is int64
+        bins = tcgs_bin_sort(cam, pr["mean2d"], pr["radius"], pr["depth"], capacity,
+                             conic=pr["conic"] if exact_tiles else None, opacity=opacity if exact_tiles else None)
+        ranges, ids = bins["tile_ranges"], bins["ids_sorted"]
+        order, counter = _training_order(cam, ranges)
+        out = tcgs_render_fwd(cam, render_opts(precision, alpha_max, tile_order=order, work_counter=counter), ranges, ids,
+                              pr["mean2d"], pr["conic"], opacity, pr["rgb"], bg=bg)
+        ctx.cam, ctx.sh_degree, ctx.alpha_max, ctx.bg = cam, sh_degree, alpha_max, bg
+        ctx.save_for_backward(means3, scales, quats, opacity, sh, pr["mean2d"], pr["conic"], pr["rgb"], pr["radius"],
+                              ranges, ids, out["img"], out["T_final"], out["n_contrib"], order)
+        ctx.mark_non_differentiable(out["T_final"])
+        return out["img"], out["T_final"]
+
+    @staticmethod
+    def backward(ctx, g_img, g_T):
+        (means3, scales, quats, opacity, sh, mean2d, conic, rgb, radius, ranges, ids, img, T_final, n_contrib,
+         order) = ctx.saved_tensors
+        needs = ctx.needs_input_grad
+        to_scene = needs[0] or needs[1] or needs[2] or needs[4]
+        P, dev = means3.shape[0], means3.device
+        shapes = [(P, 2), (P, 3), (P,), (P, 3)] + ([t.shape for t in (means3, scales, quats, sh)] if to_scene else [])
+        z = _zeros(*((s, dev) for s in shapes))   # every gradient buffer in one fill
+        g = tcgs_render_bwd(ctx.cam, render_opts("fp32", ctx.alpha_max, tile_order=order), ranges, ids, mean2d, conic,
+                            opacity, rgb, img, T_final, n_contrib, g_img.contiguous(), bg=ctx.bg,
+                            grads=dict(zip(("dmean2d", "dconic", "dopacity", "drgb"), z)))
+        p = [None] * 4
+        if to_scene:
+            p = z[4:]
+            tcgs_project_bwd(ctx.cam, means3, scales, quats, sh, ctx.sh_degree, radius, g["dmean2d"], g["dconic"],
+                             g["drgb"], grads=dict(zip(("dmeans3", "dscales", "dquats", "dsh"), p)))
+        return (p[0], p[1], p[2], g["dopacity"], p[3]) + (None,) * 8
 
 
 def render_gaussians(cam, means3, scales, quats, opacity, sh, sh_degree, precision="tc_fp16_split", alpha_max=0.99,
@@ -639,13 +677,5 @@ def render_gaussians(cam, means3, scales, quats, opacity, sh, sh_degree, precisi
     means3, scales, quats, opacity and sh through tcgs_render_bwd and tcgs_project_bwd (binning is
     piecewise constant).  Returns (img [3,H,W], T_final [H,W]).  capacity None sizes the splat
     buffer from the projection (one host synchronisation)."""
-    c = _cam(cam)
-    mean2d, conic, rgb, depth, radius, tiles = _Project.apply(means3, scales, quats, sh, c, int(sh_degree),
-                                                              opacity.detach() if tight_radius else None)
-    if capacity is None:
-        capacity = int(tiles.to(torch.int64).sum().item()) + 1
-    bins = tcgs_bin_sort(c, mean2d.detach(), radius, depth, capacity,
-                         conic=conic.detach() if exact_tiles else None,
-                         opacity=opacity.detach() if exact_tiles else None)
-    return rasterize(mean2d, conic, opacity, rgb, c, bins["tile_ranges"], bins["ids_sorted"], precision, alpha_max,
-                     bg)
+    return _RenderGaussians.apply(means3, scales, quats, opacity, sh, _cam(cam), int(sh_degree), precision, alpha_max,
+                                  tuple(bg), bool(tight_radius), capacity, bool(exact_tiles))
