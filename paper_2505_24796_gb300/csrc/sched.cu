@@ -32,8 +32,8 @@ constexpr int kFewTilesPerSm = 4;
 // One block of NT threads per tile.  Bound by the latency of two dependent gathers (id, then the
 // Gaussian's values from L2) on lists of thousands of entries, so a tile gets as many threads as keep
 // enough of them in flight: 16 views of 320 x 240 (300 tiles each, about 8000 entries a tile) took 8.13 ms
-// with one warp a tile and take 0.79 ms, which is about the sectors the gathers touch in L2 (six a list entry).
-template <int NT>
+// with one warp a tile and take 0.75 ms, bound by the gathers' requests (seven a list entry, 32 lines each).
+template <int NT, bool kPairs>
 __global__ void __launch_bounds__(NT) k_tile_features(DevCamera cam, const uint32_t* __restrict__ ranges,
                                                       const uint32_t* __restrict__ ids,
                                                       const float* __restrict__ mean2d,
@@ -63,7 +63,17 @@ __global__ void __launch_bounds__(NT) k_tile_features(DevCamera cam, const uint3
         for (int u = 0; u < kDeep; ++u) {
             o[u] = opacity[g[u]];
             d[u] = depth[g[u]];
-            a[u] = conic[3 * g[u]]; b[u] = conic[3 * g[u] + 1]; c[u] = conic[3 * g[u] + 2];
+            if (kPairs) {   // 8 bytes at the multiple of 8 inside the conic, and the other 4
+                const bool odd = g[u] & 1u;
+                const float* q = conic + 3 * (size_t)g[u];
+                const float2 two = *reinterpret_cast<const float2*>(q + (odd ? 1 : 0));
+                const float other = q[odd ? 0 : 2];
+                a[u] = odd ? other : two.x;
+                b[u] = odd ? two.x : two.y;
+                c[u] = odd ? two.y : other;
+            } else {
+                a[u] = conic[3 * (size_t)g[u]]; b[u] = conic[3 * (size_t)g[u] + 1]; c[u] = conic[3 * (size_t)g[u] + 2];
+            }
             m[u] = reinterpret_cast<const float2*>(mean2d)[g[u]];
             r[u] = (float)radius[g[u]];
         }
@@ -163,7 +173,7 @@ __global__ void __launch_bounds__(1024) k_feature_norm(const float* __restrict__
 // one 16-byte broadcast read feeds two packed FP32 operations (fma.rn.f32x2: two outputs of the same
 // input); every output's sum keeps the order bias, inputs 0 .. 31.  Read one weight at a time (and, in the
 // forward, lifted out of a loop over items into spilled registers) the two kernels took 122 us forward
-// and 129 us backward for 56,048 items; they take 12 and 32 us.
+// and 129 us backward for 56,048 items; they take 8 and 28 us.
 struct __align__(16) MlpWeights {   // FP16-rounded
     float w1[kIn][kHid], b1[kHid];  // [input][output]
     float w2[kHid][kHid + 4], b2[kHid];
@@ -171,18 +181,32 @@ struct __align__(16) MlpWeights {   // FP16-rounded
     float b3, norm[2 * kIn], pad[3];
 };
 
+// 128 threads; every load is in flight before the first store (one at a time, their latencies were 4 us of
+// either kernel).
+constexpr int kMlpThreads = 128;
+
 __device__ __forceinline__ void load_weights(const float* __restrict__ params, const float* __restrict__ norm,
                                              MlpWeights& w) {
-    for (int i = threadIdx.x; i < kParams; i += blockDim.x) {
-        const float v = h16(params[i]);
-        if (i < kB1) w.w1[i % kIn][i / kIn] = v;
-        else if (i < kW2) w.b1[i - kB1] = v;
-        else if (i < kB2) w.w2[(i - kW2) % kHid][(i - kW2) / kHid] = v;
-        else if (i < kW3) w.b2[i - kB2] = v;
-        else if (i < kB3) w.w3[i - kW3] = v;
-        else w.b3 = v;
+    constexpr int kEach = (kParams + kMlpThreads - 1) / kMlpThreads;
+    float v[kEach], nm = 0.f;
+#pragma unroll
+    for (int q = 0; q < kEach; ++q) {
+        const int i = q * kMlpThreads + threadIdx.x;
+        v[q] = i < kParams ? params[i] : 0.f;
     }
-    for (int i = threadIdx.x; i < 2 * kIn; i += blockDim.x) w.norm[i] = norm[i];
+    if (threadIdx.x < 2 * kIn) nm = norm[threadIdx.x];
+#pragma unroll
+    for (int q = 0; q < kEach; ++q) {
+        const int i = q * kMlpThreads + threadIdx.x;
+        const float x = h16(v[q]);
+        if (i < kB1) w.w1[i % kIn][i / kIn] = x;
+        else if (i < kW2) w.b1[i - kB1] = x;
+        else if (i < kB2) w.w2[(i - kW2) % kHid][(i - kW2) / kHid] = x;
+        else if (i < kW3) w.b2[i - kB2] = x;
+        else if (i < kB3) w.w3[i - kW3] = x;
+        else if (i == kB3) w.b3 = x;
+    }
+    if (threadIdx.x < 2 * kIn) w.norm[threadIdx.x] = nm;
 }
 
 // acc[0 .. 31] += in * row[0 .. 31], two outputs an operation.
@@ -233,7 +257,7 @@ __device__ __forceinline__ float mlp_forward(const MlpWeights& w, const float* _
     return y;
 }
 
-__global__ void __launch_bounds__(128) k_mlp_fwd(const float* __restrict__ params, const float* __restrict__ norm,
+__global__ void __launch_bounds__(kMlpThreads) k_mlp_fwd(const float* __restrict__ params, const float* __restrict__ norm,
                                                  const float* __restrict__ x, int n, float* __restrict__ y) {
     __shared__ MlpWeights w;
     load_weights(params, norm, w);
@@ -249,7 +273,7 @@ __global__ void __launch_bounds__(128) k_mlp_fwd(const float* __restrict__ param
 // then sums every parameter's gradient over its items, each thread a 4 x 2 piece of W2's, two of W1's and
 // one of the rest, and adds it to `grad` with one atomic each.  61 KB a block: 3 blocks an SM, so that
 // 58,000 items are one wave.
-constexpr int kBwdItems = 128;
+constexpr int kBwdItems = kMlpThreads;
 
 struct __align__(16) MlpBwdSmem {
     MlpWeights w;
@@ -281,9 +305,14 @@ __global__ void __launch_bounds__(kBwdItems) k_mlp_bwd(const float* __restrict__
     extern __shared__ __align__(16) uint8_t smem[];
     MlpBwdSmem& s = *reinterpret_cast<MlpBwdSmem*>(smem);
     load_weights(params, norm, s.w);
-    for (int i = threadIdx.x; i < kHid * kHid; i += kBwdItems) s.w2[i / kHid][i % kHid] = h16(params[kW2 + i]);
     __syncthreads();
     const int t = threadIdx.x;
+#pragma unroll
+    for (int q = 0; q < kHid * kHid / kBwdItems; ++q) {   // the weights by output, from those by input
+        const int i = q * kBwdItems + t;
+        s.w2[i / kHid][i % kHid] = s.w.w2[i % kHid][i / kHid];
+    }
+    __syncthreads();
     const int i = blockIdx.x * kBwdItems + t;
     float se = 0.f;
     if (i < n) {
@@ -379,12 +408,13 @@ extern "C" tcgs_status tcgs_tile_features(const tcgs_camera* cam, const uint32_t
     // a view of few tiles leaves most of the chip idle unless each tile gets many warps
     DeviceInfo d;
     const int sms = current_device_info(&d) ? d.sms : 128;
-    if (tiles <= kFewTilesPerSm * sms)
-        k_tile_features<512><<<tiles, 512, 0, (cudaStream_t)stream>>>(dc, tile_ranges, ids_sorted, mean2d, conic, opacity,
-                                                                      depth, radius, features);
-    else
-        k_tile_features<128><<<tiles, 128, 0, (cudaStream_t)stream>>>(dc, tile_ranges, ids_sorted, mean2d, conic, opacity,
-                                                                      depth, radius, features);
+    const bool pairs = (reinterpret_cast<uintptr_t>(conic) & 7) == 0;
+    auto launch = [&](auto kern, int threads) {
+        kern<<<tiles, threads, 0, (cudaStream_t)stream>>>(dc, tile_ranges, ids_sorted, mean2d, conic, opacity, depth, radius,
+                                                          features);
+    };
+    if (tiles <= kFewTilesPerSm * sms) pairs ? launch(k_tile_features<512, true>, 512) : launch(k_tile_features<512, false>, 512);
+    else pairs ? launch(k_tile_features<128, true>, 128) : launch(k_tile_features<128, false>, 128);
     count_launches(1);
     TCGS_CHECK_LAUNCH();
     return TCGS_OK;
