@@ -178,6 +178,14 @@ TCGS_API tcgs_status tcgs_project_bwd(const tcgs_camera* cam /* host */, int32_t
                              const float* drgb, float* dmeans3, float* dscales, float* dquats, float* dsh,
                              tcgs_stream stream);
 
+/* tcgs_project_bwd that stores the gradients (0 where radius <= 0) instead of adding to them: the same values
+ * as on zeroed arrays, without their fill. */
+TCGS_API tcgs_status tcgs_project_bwd_write(const tcgs_camera* cam /* host */, int32_t P, int32_t sh_degree,
+                             const float* means3, const float* scales, const float* quats, const float* sh,
+                             const int32_t* radius, const float* dmean2d, const float* dconic,
+                             const float* drgb, float* dmeans3, float* dscales, float* dquats, float* dsh,
+                             tcgs_stream stream);
+
 /* Bytes of device workspace tcgs_bin_sort needs (a pure host function). */
 TCGS_API size_t tcgs_bin_sort_workspace_size(int32_t P, int64_t splat_capacity, int32_t num_tiles);
 

@@ -128,14 +128,17 @@ def tcgs_project(cam, means3, scales, quats, sh, sh_degree, out=None, stream=Non
 
 def tcgs_project_bwd(cam, means3, scales, quats, sh, sh_degree, radius, dmean2d, dconic, drgb, grads=None,
                      stream=None) -> dict:
-    """Accumulates dL/d(means3, scales, quats, sh) into ``grads`` (zeros when None) and returns it."""
+    """Accumulates dL/d(means3, scales, quats, sh) into ``grads`` and returns it; with None, stores them in new
+    tensors (tcgs_project_bwd_write)."""
     c = _cam(cam)
     P = means3.shape[0]
+    fn = _L().tcgs_project_bwd
     if grads is None:
-        grads = dict(zip(("dmeans3", "dscales", "dquats", "dsh"),
-                         _zeros(*((t.shape, t.device) for t in (means3, scales, quats, sh)))))
+        grads = dict(dmeans3=torch.empty_like(means3), dscales=torch.empty_like(scales), dquats=torch.empty_like(quats),
+                     dsh=torch.empty_like(sh))
+        fn = _L().tcgs_project_bwd_write
     f = torch.float32
-    check("tcgs_project_bwd", _L().tcgs_project_bwd(
+    check("tcgs_project_bwd", fn(
         ctypes.byref(c), P, int(sh_degree), _ptr(means3, f, "means3"), _ptr(scales, f, "scales"),
         _ptr(quats, f, "quats"), _ptr(sh, f, "sh"), _ptr(radius, torch.int32, "radius"),
         _ptr(dmean2d, f, "dmean2d"), _ptr(dconic, f, "dconic"), _ptr(drgb, f, "drgb"),
@@ -656,18 +659,13 @@ class _RenderGaussians(torch.autograd.Function):
         (means3, scales, quats, opacity, sh, mean2d, conic, rgb, radius, ranges, ids, img, T_final, n_contrib,
          order) = ctx.saved_tensors
         needs = ctx.needs_input_grad
-        to_scene = needs[0] or needs[1] or needs[2] or needs[4]
-        P, dev = means3.shape[0], means3.device
-        shapes = [(P, 2), (P, 3), (P,), (P, 3)] + ([t.shape for t in (means3, scales, quats, sh)] if to_scene else [])
-        z = _zeros(*((s, dev) for s in shapes))   # every gradient buffer in one fill
         g = tcgs_render_bwd(ctx.cam, render_opts("fp32", ctx.alpha_max, tile_order=order), ranges, ids, mean2d, conic,
-                            opacity, rgb, img, T_final, n_contrib, g_img.contiguous(), bg=ctx.bg,
-                            grads=dict(zip(("dmean2d", "dconic", "dopacity", "drgb"), z)))
+                            opacity, rgb, img, T_final, n_contrib, g_img.contiguous(), bg=ctx.bg)
         p = [None] * 4
-        if to_scene:
-            p = z[4:]
-            tcgs_project_bwd(ctx.cam, means3, scales, quats, sh, ctx.sh_degree, radius, g["dmean2d"], g["dconic"],
-                             g["drgb"], grads=dict(zip(("dmeans3", "dscales", "dquats", "dsh"), p)))
+        if needs[0] or needs[1] or needs[2] or needs[4]:
+            p = tcgs_project_bwd(ctx.cam, means3, scales, quats, sh, ctx.sh_degree, radius, g["dmean2d"], g["dconic"],
+                                 g["drgb"])
+            p = [p[k] for k in ("dmeans3", "dscales", "dquats", "dsh")]
         return (p[0], p[1], p[2], g["dopacity"], p[3]) + (None,) * 8
 
 

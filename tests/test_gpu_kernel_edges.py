@@ -305,3 +305,27 @@ def test_row_lists_equal_radix_lists(tc, height, mode):
     assert int(again["status"].item()) == 3
     if mode == "rectangles":
         assert int(again["n_splats"].item()) == la.sum()
+
+
+@pytest.mark.parametrize("degree", [0, 1, 2, 3])
+def test_project_backward_store_equals_accumulate(tc, degree):
+    """Stored gradients are those added to zeroed arrays, unseen Gaussians' and whole unseen warps' included."""
+    for P, behind in ((1, 1), (33, 5), (161, 2), (100, 100)):
+        cam, sc = scenes.plain_forward(P=P, seed=50 + P)
+        rng = np.random.default_rng(P)
+        sc = dict(sc, sh=f32(rng.normal(0, 0.3, (P, (degree + 1) ** 2, 3))), sh_degree=degree)
+        sc["means3"] = sc["means3"].copy()
+        sc["means3"][::behind, 2] = -1.0
+        if P == 161:
+            sc["means3"][32:64, 2] = -1.0
+        d = tc.scene_to_device(sc, DEV)
+        pr = tc.tcgs_project(cam, d["means3"], d["scales"], d["quats"], d["sh"], degree)
+        w = [to_torch(f32(rng.normal(size=(P, k))), DEV) for k in (2, 3, 3)]
+        args = (cam, d["means3"], d["scales"], d["quats"], d["sh"], degree, pr["radius"], *w)
+        zeros = {"d" + k: torch.zeros_like(d[k]) for k in ("means3", "scales", "quats", "sh")}
+        added = tc.tcgs_project_bwd(*args, grads=zeros)
+        for _ in range(2):      # fresh memory is not zero
+            torch.full((P, 400), float("nan"), device=DEV)
+            stored = tc.tcgs_project_bwd(*args)
+            for k in added:
+                assert torch.equal(stored[k], added[k]), (P, k)
