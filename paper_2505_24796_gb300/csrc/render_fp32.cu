@@ -35,7 +35,8 @@ struct FwdParams {
 // fragment's conic form, is at least its minimum over the block's pixel centres, and alpha >= 1/255 needs
 // q <= the reach limit.  Both are compared with a slack for the rounding of q here and in the exponent
 // (kQSlack of the sum of magnitudes of its terms); conics that are not safely positive definite, and
-// values too large for the bound, are walked everywhere.
+// values too large for the bound, are walked everywhere.  1024 x 512, 250k Gaussians of small footprints: 230 us
+// with every entry at every pixel, 133 us so, 98 us with the tiles longest first.
 constexpr int kFwdThreads = kPairThreads;
 constexpr int kFwdWarps = kFwdThreads / 32;
 constexpr int kFwdBatch = kFwdThreads;
@@ -245,6 +246,9 @@ __global__ void __launch_bounds__(kFwdThreads, 7) k_render_fp32(FwdParams p) {
 //     each one by one);
 //   - the block adds its warps' sums once per batch of 128, a thread per fragment (slots that no warp replayed
 //     are not read), and issues one atomic per parameter.
+// Four blocks of 128 threads an SM (128 registers; five blocks spill, and with two fragments' exponentials at a time
+// are slower).  1024 x 512, 250k Gaussians: 403 us one fragment at a time, 263 us so, 193 us with the tiles
+// longest first; 1280 x 720, 500k wide ones: 315 and 236 us; 1920 x 1080, 1M: 732 and 583 us (515 longest first).
 // The sums over a tile are formed in a fixed order (a thread's two pixels, the butterfly's levels 16 .. 1,
 // the warps): only the order of the tiles' atomics differs between runs.
 
