@@ -43,8 +43,8 @@ constexpr int kFwdBatch = kFwdThreads;
 constexpr int kFwdGroup = 4;
 constexpr float kQSlack = 2e-6f;   // about 17 roundings
 
-// The forward's limit on q for a Gaussian at (x, y) from the tile's centre: negative when no pixel blends it,
-// infinite when the test must not be used.
+// The block tests' limit on q for a Gaussian at (x, y) from the tile's centre, the same in the forward and the
+// backward: negative when no pixel blends it, infinite when the test must not be used.
 __device__ __forceinline__ float fp32_limit(float x, float y, float a, float b, float c, float o, float lno) {
     const float inf = __int_as_float(0x7f800000);
     const float X = fabsf(x) + 0.5f * kTile, Y = fabsf(y) + 0.5f * kTile;
@@ -238,9 +238,8 @@ __global__ void __launch_bounds__(kFwdThreads, 7) k_render_fp32(FwdParams p) {
 // Hence
 //   - the two pixels of a thread go through packed FP32 instructions (fma.rn.f32x2 and its kin: one issue
 //     slot for two IEEE results), from operands staged twice over in shared memory;
-//   - a warp replays only the fragments that can reach alpha >= 1/255 somewhere in its block (the exact
-//     minimum of the conic form over the block's pixel centres against the reach limit), listed per
-//     batch of kBwdBatch fragments, four at a time: the exponentials of four fragments are independent, and
+//   - a warp replays only the fragments that the forward's block test admits (fp32_limit: with the bare reach limit,
+//     needles whose form cancels were blended by the forward and left out here), listed per batch of kBwdBatch fragments, four at a time: the exponentials of four fragments are independent, and
 //     their sums share the warp reduction: two transposing levels leave each quarter of the warp with one
 //     fragment's nine sums over eight lanes, three more finish them (37 shuffles for four fragments; 14
 //     each one by one);
@@ -294,7 +293,7 @@ __global__ void __launch_bounds__(kBwdThreads, 4) k_render_bwd(BwdParams p) {
     const PairPixels q = pair_pixels(warp, lane);
     const float cx = (float)(tx * kTile + kTile / 2), cy = (float)(ty * kTile + kTile / 2);
     const uint32_t start = p.ranges[2 * tile], end = p.ranges[2 * tile + 1];
-    const float amax = p.alpha_max;
+    const float amax = p.alpha_max, inf = __int_as_float(0x7f800000);
 
     // per pixel: n_contrib, -dL/dimg, T_final, the colour still to come, the replayed T
     uint32_t nc[2] = {0u, 0u};
@@ -347,7 +346,7 @@ __global__ void __launch_bounds__(kBwdThreads, 4) k_render_bwd(BwdParams p) {
         if (valid) {
             const float2 m = reinterpret_cast<const float2*>(p.mean2d)[g];
             const float a = p.conic[3 * (size_t)g], b = p.conic[3 * (size_t)g + 1], c = p.conic[3 * (size_t)g + 2], o = p.opacity[g];
-            const float lno = __logf(o), lim = reach_limit(lno);
+            const float lno = __logf(o), lim = fp32_limit(m.x - cx, m.y - cy, a, b, c, o, lno);
             const float r = p.rgb[3 * (size_t)g], gr = p.rgb[3 * (size_t)g + 1], bl = p.rgb[3 * (size_t)g + 2];
             s_f[t] = pair_rec(m.x, m.y, a, b, c, o, r, gr, bl, lno);
             odd = odd || !(fabsf(r) + fabsf(gr) + fabsf(bl) < kHuge);
@@ -356,7 +355,7 @@ __global__ void __launch_bounds__(kBwdThreads, 4) k_render_bwd(BwdParams p) {
 #pragma unroll
                 for (int k = 0; k < kBwdWarps; ++k) {
                     const float x0 = 8.f * (k & 1) - 7.5f, y0 = 8.f * (k >> 1) - 7.5f;
-                    near_[k] = min_q_box_facing(m.x - cx, m.y - cy, a, b, c, ia, ic, x0, x0 + 7.f, y0, y0 + 7.f) <= lim;
+                    near_[k] = lim == inf || min_q_box_facing(m.x - cx, m.y - cy, a, b, c, ia, ic, x0, x0 + 7.f, y0, y0 + 7.f) <= lim;
                 }
             }
         }

@@ -1,0 +1,65 @@
+"""Inputs at the limits of what the kernels' shortcuts may assume: needles, conics that are no ellipse, infinities,
+oversized arrays, ill-formed lists."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2505_24796_gb300 import scenes
+
+from .helpers import f32, to_torch
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+@pytest.fixture(scope="module")
+def tc():
+    import paper_2505_24796_gb300 as m
+    m._lib.load()
+    return m
+
+
+def _needle_conics(rng, sigma_long, n):
+    """FP32 conics of needles `sigma_long` pixels long (n values) and under two wide, with the 0.3 px dilation, and the
+    unit vectors along them."""
+    s, th = rng.uniform(0.3, 2.0, n), rng.uniform(0, np.pi, n)
+    c, d = np.cos(th), np.sin(th)
+    A, B, C = ((c * sigma_long) ** 2 + (d * s) ** 2 + 0.3, c * d * (sigma_long ** 2 - s ** 2),
+               (d * sigma_long) ** 2 + (c * s) ** 2 + 0.3)
+    return f32(np.stack([C, -B, A], 1) / (A * C - B * B)[:, None]), np.stack([c, d], 1)
+
+
+@pytest.mark.parametrize("kind", ["needles_100_400", "needles_500_1500", "hyperbolic", "nan"])
+@pytest.mark.parametrize("early", [False, True])
+def test_backward_replays_what_the_forward_blended(tc, kind, early):
+    """One Gaussian a tile, of colour 1: the image is its alpha, and with dL/dimg = 1 in one channel its colour
+    gradient is the sum of the tile's pixels (256 positive terms added by a tree of at most 12 roundings: 1e-6).
+    Needles whose means lie 2 to 3.4 sigma along their axis from the tile, where the conic form cancels, and
+    conics that are no ellipse."""
+    rng = np.random.default_rng(len(kind))
+    gw = gh = 64
+    n = gw * gh
+    cam = scenes.pinhole(16 * gw, 16 * gh, fx=500.0)
+    centre = np.stack([np.arange(n) % gw, np.arange(n) // gw], 1) * 16.0 + 8.0
+    if kind.startswith("needles"):
+        lo, hi = (float(v) for v in kind.split("_")[1:])
+        L = rng.uniform(lo, hi, n)
+        conic, axis = _needle_conics(rng, L, n)
+        mean2d = f32(centre + axis * (rng.choice([-1, 1], n) * rng.uniform(2, 3.4, n) * L)[:, None] + rng.uniform(-6, 6, (n, 2)))
+    else:
+        mean2d = f32(centre + rng.uniform(-40, 40, (n, 2)))
+        conic = f32(np.tile([0.01, 0.5, 0.01] if kind == "hyperbolic" else [np.nan, 0.1, 0.2], (n, 1)))
+    t = {k: to_torch(v, DEV) for k, v in dict(mean2d=mean2d, conic=conic, opacity=f32(rng.uniform(0.5, 0.99, n)),
+                                              rgb=np.ones((n, 3), np.float32)).items()}
+    ids = torch.arange(n, dtype=torch.int32, device=DEV)
+    ranges = torch.stack([ids, ids + 1], 1).contiguous()
+    opts = tc.render_opts("fp32", early_cull=early)
+    args = (t["mean2d"], t["conic"], t["opacity"], t["rgb"])
+    o = tc.tcgs_render_fwd(cam, opts, ranges, ids, *args)
+    dl = torch.zeros_like(o["img"])
+    dl[0] = 1
+    g = tc.tcgs_render_bwd(cam, opts, ranges, ids, *args, o["img"], o["T_final"], o["n_contrib"], dl)
+    alpha = o["img"][0].double().view(gh, 16, gw, 16).sum(dim=(1, 3)).view(-1)
+    assert int((alpha > 0).sum()) > n // 20
+    torch.testing.assert_close(g["drgb"][:, 0].double(), alpha, rtol=1e-6, atol=0)
