@@ -349,7 +349,8 @@ __global__ void __launch_bounds__(kBwdThreads, 4) k_render_bwd(BwdParams p) {
             const float lno = __logf(o), lim = fp32_limit(m.x - cx, m.y - cy, a, b, c, o, lno);
             const float r = p.rgb[3 * (size_t)g], gr = p.rgb[3 * (size_t)g + 1], bl = p.rgb[3 * (size_t)g + 2];
             s_f[t] = pair_rec(m.x, m.y, a, b, c, o, r, gr, bl, lno);
-            odd = odd || !(fabsf(r) + fabsf(gr) + fabsf(bl) < kHuge);
+            odd = odd || !(fabsf(r) + fabsf(gr) + fabsf(bl) < kHuge) || !(fabsf(a) + fabsf(b) + fabsf(c) < kHuge) ||
+                  !(fabsf(m.x) + fabsf(m.y) < kHuge);
             if (lim >= 0.f) {
                 const float ia = __fdividef(1.f, a), ic = __fdividef(1.f, c);
 #pragma unroll
@@ -421,7 +422,8 @@ __global__ void __launch_bounds__(kBwdThreads, 4) k_render_bwd(BwdParams p) {
                 float v[2][kBwdParams];
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
-                    const f32x2 na_f = na[f + e], G_f = G[f + e], dx_f = dx[f + e], dy_f = dy[f + e];
+                    const f32x2 na_f = na[f + e], G_f = G[f + e];
+                    f32x2 dx_f = dx[f + e], dy_f = dy[f + e];
                     const PairRec& r = s_f[(four >> (8 * (f + e))) & 0xFFu];
                     f32x2 cr = r.q[3].x, cg = r.q[3].y, cb = r.q[4].x, h0 = ng0, h1 = ng1, h2 = ng2;
                     if (strict) {   // 0 times an infinity or a NaN would reach what does not blend it
@@ -449,8 +451,12 @@ __global__ void __launch_bounds__(kBwdThreads, 4) k_render_bwd(BwdParams p) {
                     const f32x2 nd = where2(G_f, nd_all);
                     const f32x2 d = mul2(nd, na_f);   // dL/dpower
                     const f32x2 bx = mul2(r.q[1].x, dx_f), cy = mul2(r.q[1].y, dy_f);
-                    const f32x2 m0 = fma2(r.q[1].x, dy_f, mul2(r.q[0].y, dx_f));   // -(a dx + b dy)
-                    const f32x2 m1 = pack2f(__fadd_rn(lo2(bx), lo2(cy)), __fadd_rn(hi2(bx), hi2(cy)));   // -(b dx + c dy)
+                    f32x2 m0 = fma2(r.q[1].x, dy_f, mul2(r.q[0].y, dx_f));   // -(a dx + b dy)
+                    f32x2 m1 = pack2f(__fadd_rn(lo2(bx), lo2(cy)), __fadd_rn(hi2(bx), hi2(cy)));   // -(b dx + c dy)
+                    if (strict) {   // nor may the geometry's, where d is 0
+                        m0 = where2(G_f, m0); m1 = where2(G_f, m1);
+                        dx_f = where2(G_f, dx_f); dy_f = where2(G_f, dy_f);
+                    }
                     const f32x2 ddx = mul2(d, dx_f), ddy = mul2(d, dy_f);
                     v[e][0] = dot2(d, m0);
                     v[e][1] = dot2(d, m1);

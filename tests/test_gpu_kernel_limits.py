@@ -63,3 +63,32 @@ def test_backward_replays_what_the_forward_blended(tc, kind, early):
     alpha = o["img"][0].double().view(gh, 16, gw, 16).sum(dim=(1, 3)).view(-1)
     assert int((alpha > 0).sum()) > n // 20
     torch.testing.assert_close(g["drgb"][:, 0].double(), alpha, rtol=1e-6, atol=0)
+
+
+@pytest.mark.parametrize("conic,mean", [((3e37, 0, 3e37), None), ((np.inf, 0, np.inf), None), ((np.nan, 0.1, 0.2), None),
+                                        (None, (np.inf, 8)), (None, (8, -np.inf)), (None, (np.nan, 8)), (None, (3e38, 3e38))])
+def test_backward_keeps_odd_geometry_where_it_is_not_blended(tc, conic, mean):
+    """A conic that overflows at a pixel's offset, an infinity or a NaN in a conic or a mean: a pixel that does not
+    blend the Gaussian, or blends it with a clamped alpha, adds nothing to the gradients of its geometry, and every
+    other Gaussian's gradients stay finite."""
+    rng = np.random.default_rng(2)
+    n, cam = 24, scenes.pinhole(16, 16, fx=50.0)
+    s = rng.uniform(2, 6, n)
+    inp = dict(mean2d=f32(rng.uniform(0, 16, (n, 2))), conic=f32(np.stack([1 / s ** 2, 0 * s, 1 / s ** 2], 1)),
+               opacity=f32(rng.uniform(0.05, 0.3, n)), rgb=f32(rng.uniform(0, 1, (n, 3))))
+    inp["mean2d"][9] = 8
+    if conic is not None:
+        inp["conic"][9] = f32(conic)
+    if mean is not None:
+        inp["mean2d"][9] = f32(mean)
+    t = [to_torch(inp[k], DEV) for k in ("mean2d", "conic", "opacity", "rgb")]
+    ids = torch.arange(n, dtype=torch.int32, device=DEV)
+    ranges = torch.tensor([[0, n]], dtype=torch.int32, device=DEV)
+    o = tc.tcgs_render_fwd(cam, tc.render_opts("fp32"), ranges, ids, *t)
+    g = tc.tcgs_render_bwd(cam, tc.render_opts("fp32"), ranges, ids, *t, o["img"], o["T_final"], o["n_contrib"],
+                           to_torch(f32(rng.standard_normal((3, 16, 16))), DEV))
+    assert int(o["n_contrib"].max()) > 10
+    for k, v in g.items():
+        assert torch.isfinite(v).all(), k
+    for k in ("dmean2d", "dconic", "dopacity"):
+        assert (g[k][9] == 0).all(), k
