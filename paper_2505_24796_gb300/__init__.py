@@ -134,9 +134,11 @@ def tcgs_project_bwd(cam, means3, scales, quats, sh, sh_degree, radius, dmean2d,
     P = means3.shape[0]
     fn = _L().tcgs_project_bwd
     if grads is None:
-        grads = dict(dmeans3=torch.empty_like(means3), dscales=torch.empty_like(scales), dquats=torch.empty_like(quats),
-                     dsh=torch.empty_like(sh))
-        fn = _L().tcgs_project_bwd_write
+        new = torch.zeros_like   # an array with rows beyond P, which the call does not write
+        if (means3.numel(), scales.numel(), quats.numel(), sh.numel()) == (
+                3 * P, 3 * P, 4 * P, 3 * (int(sh_degree) + 1) ** 2 * P):
+            new, fn = torch.empty_like, _L().tcgs_project_bwd_write
+        grads = dict(dmeans3=new(means3), dscales=new(scales), dquats=new(quats), dsh=new(sh))
     f = torch.float32
     check("tcgs_project_bwd", fn(
         ctypes.byref(c), P, int(sh_degree), _ptr(means3, f, "means3"), _ptr(scales, f, "scales"),

@@ -92,3 +92,19 @@ def test_backward_keeps_odd_geometry_where_it_is_not_blended(tc, conic, mean):
         assert torch.isfinite(v).all(), k
     for k in ("dmean2d", "dconic", "dopacity"):
         assert (g[k][9] == 0).all(), k
+
+
+@pytest.mark.parametrize("extra", ["sh", "scales", "quats"])
+def test_project_backward_zeroes_rows_beyond_its_gaussians(tc, monkeypatch, extra):
+    """Arrays with more rows than there are Gaussians: the rows that belong to none get a gradient of 0, whatever
+    the memory held."""
+    cam, sc = scenes.plain_forward(P=40, seed=3)
+    d = tc.scene_to_device(sc, DEV)
+    pr = tc.tcgs_project(cam, d["means3"], d["scales"], d["quats"], d["sh"], d["sh_degree"])
+    d[extra] = torch.cat([d[extra], torch.ones_like(d[extra])])
+    w = [torch.randn(40, k, device=DEV) for k in (2, 3, 3)]
+    monkeypatch.setattr(torch, "empty_like", lambda t: torch.full_like(t, float("nan")))
+    g = tc.tcgs_project_bwd(cam, d["means3"], d["scales"], d["quats"], d["sh"], d["sh_degree"], pr["radius"], *w)
+    assert (g["d" + extra][40:] == 0).all()
+    for k, v in g.items():
+        assert torch.isfinite(v).all() and (v[:40] != 0).any(), k
