@@ -65,8 +65,8 @@ def test_backward_replays_what_the_forward_blended(tc, kind, early):
     torch.testing.assert_close(g["drgb"][:, 0].double(), alpha, rtol=1e-6, atol=0)
 
 
-@pytest.mark.parametrize("conic,mean", [((3e37, 0, 3e37), None), ((np.inf, 0, np.inf), None), ((np.nan, 0.1, 0.2), None),
-                                        (None, (np.inf, 8)), (None, (8, -np.inf)), (None, (np.nan, 8)), (None, (3e38, 3e38))])
+@pytest.mark.parametrize("conic,mean", [((1e38, 0, 1e38), None), ((np.inf, 0, np.inf), None), ((np.nan, 0.1, 0.2), None),
+                                        (None, (np.inf, 4)), (None, (4, -np.inf)), (None, (np.nan, 4)), (None, (3e38, 3e38))])
 def test_backward_keeps_odd_geometry_where_it_is_not_blended(tc, conic, mean):
     """A conic that overflows at a pixel's offset, an infinity or a NaN in a conic or a mean: a pixel that does not
     blend the Gaussian, or blends it with a clamped alpha, adds nothing to the gradients of its geometry, and every
@@ -76,7 +76,7 @@ def test_backward_keeps_odd_geometry_where_it_is_not_blended(tc, conic, mean):
     s = rng.uniform(2, 6, n)
     inp = dict(mean2d=f32(rng.uniform(0, 16, (n, 2))), conic=f32(np.stack([1 / s ** 2, 0 * s, 1 / s ** 2], 1)),
                opacity=f32(rng.uniform(0.05, 0.3, n)), rgb=f32(rng.uniform(0, 1, (n, 3))))
-    inp["mean2d"][9] = 8
+    inp["mean2d"][9] = 4    # between the pixel centres of the first block
     if conic is not None:
         inp["conic"][9] = f32(conic)
     if mean is not None:
