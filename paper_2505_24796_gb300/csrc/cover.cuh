@@ -74,9 +74,10 @@ __device__ __forceinline__ bool tile_reached(const Cover& v, float lx, float ly)
 // the same band of rows, and a box meets the convex region {q <= lim} exactly when its x-range meets
 // the region's shadow on the x axis within that band.  So each (Gaussian, tile row) is one unit of
 // work: the shadow's ends come from the ellipse in closed form, and the per-tile test (tile_reached)
-// fixes the interval's end tiles, so the tiles kept are those the per-tile test keeps (whenever they
-// form one run, which they do up to FP32 ties at the reach limit).  Narrow rows and degenerate
-// conics test every tile of the row and keep the run from the first to the last passing tile.
+// fixes the end tiles that the closed form leaves in doubt.  row_span keeps the run from the first to the last
+// tile so found, and scans the rows of degenerate conics; row_tiles leaves every tile in doubt to the caller's
+// tests, so that the tiles are those that the per-tile test keeps, also where FP32 ties at the reach limit
+// make it keep a row in parts.
 
 // Extent of the reach ellipse {q <= lim} about the mean: half-widths W (x) and H (y), the y offset s
 // of its leftmost point (the rightmost one is at -s), and det = ac - b^2.  W < 0: scan the row.
@@ -104,6 +105,39 @@ __device__ __forceinline__ int clamp_tile(float f, int lo, int hi) {
     return (int)fminf(fmaxf(f, (float)lo), (float)hi);   // NaN -> lo
 }
 
+// The shadow [xa, xb] of the ellipse on the x axis within tile row ty's band [yl, yh] of pixel centres, relative to
+// the mean (in: the band meets the ellipse); rl and rr: half the slope of the form across its ends, at the offsets
+// dl and dr where the ellipse reaches furthest inside the band.
+struct Shadow {
+    float yl, yh, xa, xb, rl, rr;
+    bool in;
+};
+
+__device__ __forceinline__ Shadow shadow_of(const Cover& v, const Reach& e, int ty) {
+    Shadow h;
+    h.yl = __fsub_rn((float)(ty * kTile) + 0.5f, v.my);
+    h.yh = __fadd_rn(h.yl, 15.f);
+    h.xa = h.xb = h.rl = h.rr = 0.f;
+    h.in = !(h.yl > e.H || h.yh < -e.H);
+    if (h.in) {
+        const float alim = __fmul_rn(v.a, v.lim);
+        const float dl = fminf(h.yh, fmaxf(h.yl, e.s)), dr = fminf(h.yh, fmaxf(h.yl, -e.s));
+        h.rl = __fsqrt_rn(fmaxf(0.f, __fsub_rn(alim, __fmul_rn(e.det, __fmul_rn(dl, dl)))));
+        h.rr = __fsqrt_rn(fmaxf(0.f, __fsub_rn(alim, __fmul_rn(e.det, __fmul_rn(dr, dr)))));
+        h.xa = __fmul_rn(__fsub_rn(__fmul_rn(-v.b, dl), h.rl), v.ia);
+        h.xb = __fmul_rn(__fadd_rn(__fmul_rn(-v.b, dr), h.rr), v.ia);
+    }
+    return h;
+}
+
+// First and last tile whose box [16 tx + 0.5, 16 tx + 15.5] meets [mx + xa, mx + xb].
+__device__ __forceinline__ float first_met(const Cover& v, float xa) {
+    return ceilf(__fmul_rn(__fsub_rn(__fadd_rn(v.mx, xa), 15.5f), 1.f / kTile));
+}
+__device__ __forceinline__ float last_met(const Cover& v, float xb) {
+    return floorf(__fmul_rn(__fsub_rn(__fadd_rn(v.mx, xb), 0.5f), 1.f / kTile));
+}
+
 // Tiles [L, R] (empty when L > R) of rectangle columns [x0, x1] in tile row ty that Gaussian v reaches.
 __device__ int2 row_span(const Cover& v, const Reach& e, int ty, int x0, int x1) {
     const int2 none = make_int2(1, 0);
@@ -119,22 +153,9 @@ __device__ int2 row_span(const Cover& v, const Reach& e, int ty, int x0, int x1)
         return make_int2(L, R);
     };
     if (e.W < 0.f || x1 - x0 < 3) return scan();
-    // the shadow [xa, xb] of the ellipse on the x axis within the row's band of pixel centres
-    const float yl = __fsub_rn((float)(ty * kTile) + 0.5f, v.my), yh = __fadd_rn(yl, 15.f);
-    float Lf = 1.f, Rf = 0.f;   // empty unless the band meets the ellipse
-    float xa_ = 0.f, xb_ = 0.f, rl_ = 0.f, rr_ = 0.f;
-    if (!(yl > e.H || yh < -e.H)) {
-        const float alim = __fmul_rn(v.a, v.lim);
-        const float dl = fminf(yh, fmaxf(yl, e.s)), dr = fminf(yh, fmaxf(yl, -e.s));
-        const float rl = __fsqrt_rn(fmaxf(0.f, __fsub_rn(alim, __fmul_rn(e.det, __fmul_rn(dl, dl)))));
-        const float rr = __fsqrt_rn(fmaxf(0.f, __fsub_rn(alim, __fmul_rn(e.det, __fmul_rn(dr, dr)))));
-        const float xa = __fmul_rn(__fsub_rn(__fmul_rn(-v.b, dl), rl), v.ia);
-        const float xb = __fmul_rn(__fadd_rn(__fmul_rn(-v.b, dr), rr), v.ia);
-        xa_ = xa; xb_ = xb; rl_ = rl; rr_ = rr;
-        // tiles whose box [16 tx + 0.5, 16 tx + 15.5] meets [mx + xa, mx + xb]
-        Lf = ceilf(__fmul_rn(__fsub_rn(__fadd_rn(v.mx, xa), 15.5f), 1.f / kTile));
-        Rf = floorf(__fmul_rn(__fsub_rn(__fadd_rn(v.mx, xb), 0.5f), 1.f / kTile));
-    }
+    const Shadow h = shadow_of(v, e, ty);
+    const float yl = h.yl, yh = h.yh, xa_ = h.xa, xb_ = h.xb, rl_ = h.rl, rr_ = h.rr;
+    const float Lf = h.in ? first_met(v, xa_) : 1.f, Rf = h.in ? last_met(v, xb_) : 0.f;   // empty unless the band meets the ellipse
     if (!(Lf <= Rf) || Rf < (float)x0 || Lf > (float)x1) {
         // no shadow in the rectangle: probe the tile holding the point of least q in the band (the
         // least of the minima over x, (det / a) dy^2, is at the dy nearest to 0), grow from there
@@ -184,11 +205,82 @@ __device__ int2 row_span(const Cover& v, const Reach& e, int ty, int x0, int x1)
     return make_int2(L, R);
 }
 
+// Bound on the relative error of Reach.s: that of the determinant is 1.2e-7 ac / det, of which the ellipse's width
+// takes half; infinite where the terms of higher order would count.
+__device__ __forceinline__ float turn_error(const Cover& v) {
+    const float rel = 2e-7f * __fdividef(v.a * v.c, __fsub_rn(__fmul_rn(v.a, v.c), __fmul_rn(v.b, v.b)));
+    return rel >= 0.f && rel < 0.2f ? rel : __int_as_float(0x7f800000);
+}
+
+// What the closed form must clear before a tile needs no test.  Along y = dl (dr) the form is lim - 2 r e + a e^2
+// at a distance e inside the shadow's end, so the end tile passes when that is below lim at the point of its
+// box nearest to the minimum; at a distance g outside, where the outer neighbour's box begins, it is at
+// least lim + 2 (r - |b| d) g - c d^2 over the band, d being the error of dl.  Both are compared with a bound on the roundings
+// of this code and of the test: 1e-5 of the sum of magnitudes (168 times 2^-24) and of the positions.
+struct Slack {
+    float form, pos, turn;   // of the form, of a position, of half a slope (|b| d)
+    __device__ __forceinline__ float at(float r) const { return form + pos * r; }
+    __device__ __forceinline__ float slope(float r) const { return r - turn; }   // at most 0: nothing is known
+};
+
+__device__ __forceinline__ Slack slack_of(const Cover& v, float rel, const Shadow& h, float X) {
+    const float Y = fmaxf(fabsf(h.yl), fabsf(h.yh)), d = rel * Y;
+    Slack s;
+    s.form = 1e-5f * (v.a * X * X + v.c * Y * Y) + v.c * d * d;
+    s.pos = 1e-5f * (fabsf(v.mx) + X);
+    s.turn = fabsf(v.b) * d;
+    return s;
+}
+
+// far: from the shadow's end to the far side of the end tile's box.  clamped: the rectangle ends at that tile.
+__device__ __forceinline__ bool end_sure(const Cover& v, const Slack& s, float r, float far, bool clamped) {
+    const float e = fminf(fmaxf(r * v.ia, far - 15.f), far);
+    return far >= 0.f && e * (2.f * r - v.a * e) > s.at(r) && (clamped || 2.f * s.slope(r) * (16.f - far) > s.at(r));
+}
+
+// The tiles of rectangle columns [x0, x1] in tile row ty that tile_reached admits one by one, rounding included:
+// sure, exactly [lo, hi] (none when lo > hi); else some of [lo, hi], which the caller tests.  The form is
+// convex, so a row whose ends clear the slack of the whole rectangle (that of the largest offsets in it) has no
+// tile inside that fails and none outside that passes.  Needles, whose form cancels, do not clear it.
+struct RowTiles {
+    int lo, hi;
+    bool sure;
+};
+
+__device__ RowTiles row_tiles(const Cover& v, const Reach& e, float rel, int ty, int x0, int x1) {
+    const RowTiles none{1, 0, true}, all{x0, x1, false};
+    if (!(v.ia < 1e30f) || !(v.ic < 1e30f)) return all;
+    const Shadow h = shadow_of(v, e, ty);
+    const float Xl = v.mx - (float)(x0 * kTile), Xr = (float)((x1 + 1) * kTile) - v.mx;
+    const Slack s = slack_of(v, rel, h, fmaxf(fabsf(Xl), fabsf(Xr)));
+    if (!h.in) {   // the least q of the band, (det / a) dy^2, against the limit
+        const float dy = fminf(h.yh, fmaxf(h.yl, 0.f));
+        return e.det * v.ia * dy * dy > v.lim + s.form ? none : all;
+    }
+    const float Lf = first_met(v, h.xa), Rf = last_met(v, h.xb);
+    if (Rf < (float)x0)
+        return 2.f * s.slope(h.rr) * ((float)(x0 * kTile) + 0.5f - (v.mx + h.xb)) > s.at(h.rr) ? none : all;
+    if (Lf > (float)x1)
+        return 2.f * s.slope(h.rl) * ((v.mx + h.xa) - ((float)(x1 * kTile) + 15.5f)) > s.at(h.rl) ? none : all;
+    if (!(Lf <= Rf)) return all;
+    const int L = clamp_tile(Lf, x0, x1), R = clamp_tile(Rf, x0, x1);
+    if (end_sure(v, s, h.rl, (float)(L * kTile) + 15.5f - (v.mx + h.xa), (float)L > Lf) &&
+        end_sure(v, s, h.rr, (v.mx + h.xb) - ((float)(R * kTile) + 0.5f), (float)R < Rf))
+        return RowTiles{L, R, true};
+    // no tile passes beyond a distance of s.at / (2 s.slope) from the ends
+    const float ul = 2.f * s.slope(h.rl), ur = 2.f * s.slope(h.rr);
+    RowTiles t = all;
+    if (s.at(h.rl) < 1e6f * ul) t.lo = clamp_tile(first_met(v, h.xa - __fdividef(s.at(h.rl), ul)) - 1.f, x0, x1);
+    if (s.at(h.rr) < 1e6f * ur) t.hi = clamp_tile(last_met(v, h.xb + __fdividef(s.at(h.rr), ur)) + 1.f, x0, x1);
+    return t;
+}
+
 // Gaussians whose rectangle is at least this many tiles wide are covered by rows; the narrower ones
 // tile by tile (for them a row costs about as many box tests as it has tiles, plus the row's own
 // bookkeeping).
 constexpr int kRowMinWidth = 6;
-// The row path runs when the caller's splat capacity allows at least this many splats per Gaussian.
+// With a splat capacity of at least this many splats per Gaussian, wide Gaussians' rows are kept from the first
+// to the last reached tile (row_span), else tile by tile.
 constexpr int kRowsCapacityPerGaussian = 32;
 
 }  // namespace

@@ -108,3 +108,39 @@ def test_project_backward_zeroes_rows_beyond_its_gaussians(tc, monkeypatch, extr
     assert (g["d" + extra][40:] == 0).all()
     for k, v in g.items():
         assert torch.isfinite(v).all() and (v[:40] != 0).any(), k
+
+
+def _lists(o, gw, cols):
+    """Lengths and concatenated ids of the lists of the first `cols` of `gw` tile columns."""
+    r = o["tile_ranges"].long().view(-1, gw, 2)[:, :cols].reshape(-1, 2)
+    lens = r[:, 1] - r[:, 0]
+    at = torch.repeat_interleave(r[:, 0] - (lens.cumsum(0) - lens), lens) + torch.arange(int(lens.sum()), device=DEV)
+    return lens, o["ids_sorted"][at]
+
+
+@pytest.mark.parametrize("kind", ["needles", "undilated", "axis", "round"])
+def test_row_lists_of_needles_equal_radix_lists(tc, kind):
+    """Exact coverage tile by tile (fewer than 32 splats of capacity a Gaussian): a view of 256 tile columns, sorted by
+    row lists, keeps the tiles of one of 257, whose radix passes test every tile of every rectangle, also for needles
+    whose conic form cancels and whose rows are reached in parts."""
+    rng = np.random.default_rng(len(kind))
+    P, seen, H = 500_000, 60_000, 1024
+    L = np.exp(rng.uniform(*np.log([20, 60] if kind == "round" else [100, 1500]), seen))
+    s = dict(needles=rng.uniform(0.3, 2, seen), undilated=rng.uniform(1e-3, 0.2, seen), axis=rng.uniform(0.3, 2, seen),
+             round=0.8 * L)[kind]
+    th = rng.uniform(-0.01, 0.01, seen) + np.pi / 2 * rng.integers(0, 2, seen) if kind == "axis" else rng.uniform(0, np.pi, seen)
+    c, d, dil = np.cos(th), np.sin(th), 0.0 if kind == "undilated" else 0.3
+    A, B, C = f32((c * L) ** 2 + (d * s) ** 2 + dil), f32(c * d * (L * L - s * s)), f32((d * L) ** 2 + (c * s) ** 2 + dil)
+    det = A * C - B * B
+    pad = lambda a, v: np.concatenate([f32(a), np.full((P - seen,) + a.shape[1:], v, np.float32)])  # noqa: E731
+    conic = pad(np.stack([C, -B, A], 1) / np.where(det > 0, det, 1)[:, None], 1.0)
+    mean2d = pad(np.stack([rng.uniform(-50, 3000, seen), rng.uniform(-50, H + 50, seen)], 1), 0.0)
+    radius = np.zeros(P, np.int32)
+    radius[:seen] = np.where(det > 0, np.minimum(np.ceil(3 * L), 1000), 0)
+    t = [to_torch(v, DEV) for v in (mean2d, radius, f32(rng.integers(1, 500, P)))]
+    exact = dict(conic=to_torch(conic, DEV), opacity=to_torch(pad(rng.uniform(0.003, 1, seen), 1.0), DEV))
+    res = [tc.tcgs_bin_sort(scenes.pinhole(16 * gw, H, fx=500.0), *t, 32 * P - 1, **exact) for gw in (256, 257)]
+    assert [int(o["status"].item()) for o in res] == [0, 0]
+    (la, ia), (lb, ib) = _lists(res[0], 256, 256), _lists(res[1], 257, 256)
+    assert int(la.sum()) == int(res[0]["n_splats"].item())
+    assert int((la != lb).sum()) == 0 and torch.equal(ia, ib)
