@@ -66,7 +66,8 @@ __global__ void __launch_bounds__(kFwdThreads, 7) k_render_fp32(FwdParams p) {
     const int tx = tile % p.cam.grid_w, ty = tile / p.cam.grid_w;
     const PairPixels q = pair_pixels(warp, lane);
     const float cx = (float)(tx * kTile + kTile / 2), cy = (float)(ty * kTile + kTile / 2);
-    const uint32_t start = p.ranges[2 * tile], len = p.ranges[2 * tile + 1] - start;
+    const uint32_t start = p.ranges[2 * tile], stop = p.ranges[2 * tile + 1];
+    const uint32_t len = stop > start ? stop - start : 0u;   // an inverted range is an empty list
     const float amax = p.alpha_max, inf = __int_as_float(0x7f800000);
     const int px_i = tx * kTile + q.lx, py_i = ty * kTile + q.ly;
     const bool in0 = px_i < p.cam.width && py_i < p.cam.height, in1 = px_i < p.cam.width && py_i + 4 < p.cam.height;
@@ -239,7 +240,8 @@ __global__ void __launch_bounds__(kFwdThreads, 7) k_render_fp32(FwdParams p) {
 //   - the two pixels of a thread go through packed FP32 instructions (fma.rn.f32x2 and its kin: one issue
 //     slot for two IEEE results), from operands staged twice over in shared memory;
 //   - a warp replays only the fragments that the forward's block test admits (fp32_limit: with the bare reach limit,
-//     needles whose form cancels were blended by the forward and left out here), listed per batch of kBwdBatch fragments, four at a time: the exponentials of four fragments are independent, and
+//     needles whose form cancels were blended by the forward and left out here), listed per batch of
+//     kBwdBatch fragments, four at a time: the exponentials of four fragments are independent, and
 //     their sums share the warp reduction: two transposing levels leave each quarter of the warp with one
 //     fragment's nine sums over eight lanes, three more finish them (37 shuffles for four fragments; 14
 //     each one by one);
@@ -292,7 +294,8 @@ __global__ void __launch_bounds__(kBwdThreads, 4) k_render_bwd(BwdParams p) {
     const int tx = tile % p.cam.grid_w, ty = tile / p.cam.grid_w;
     const PairPixels q = pair_pixels(warp, lane);
     const float cx = (float)(tx * kTile + kTile / 2), cy = (float)(ty * kTile + kTile / 2);
-    const uint32_t start = p.ranges[2 * tile], end = p.ranges[2 * tile + 1];
+    const uint32_t start = p.ranges[2 * tile], stop = p.ranges[2 * tile + 1];
+    const uint32_t end = stop > start ? stop : start;   // an inverted range is an empty list
     const float amax = p.alpha_max, inf = __int_as_float(0x7f800000);
 
     // per pixel: n_contrib, -dL/dimg, T_final, the colour still to come, the replayed T

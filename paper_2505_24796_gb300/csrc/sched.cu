@@ -47,7 +47,8 @@ __global__ void __launch_bounds__(NT) k_tile_features(DevCamera cam, const uint3
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int tx = tile % cam.grid_w, ty = tile / cam.grid_w;
     const float x0 = (float)(kTile * tx), y0 = (float)(kTile * ty);
-    const uint32_t start = ranges[2 * tile], end = ranges[2 * tile + 1], len = end - start;
+    const uint32_t start = ranges[2 * tile], end = ranges[2 * tile + 1];
+    const uint32_t len = end > start ? end - start : 0u;   // an inverted range is an empty list
     float so = 0.f, mo = 0.f, dmin = 3.0e38f, dmax = -3.0e38f, sdet = 0.f, cov = 0.f;
     for (uint32_t k0 = threadIdx.x; k0 < len; k0 += kDeep * NT) {
         uint32_t g[kDeep];

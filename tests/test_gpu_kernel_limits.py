@@ -144,3 +144,24 @@ def test_row_lists_of_needles_equal_radix_lists(tc, kind):
     (la, ia), (lb, ib) = _lists(res[0], 256, 256), _lists(res[1], 257, 256)
     assert int(la.sum()) == int(res[0]["n_splats"].item())
     assert int((la != lb).sum()) == 0 and torch.equal(ia, ib)
+
+
+def test_inverted_ranges_are_empty_lists(tc):
+    """A range whose end lies before its start holds no entry: background, no gradient, an empty list's features."""
+    cam = scenes.pinhole(48, 32, fx=50.0)
+    n = 40
+    rng = np.random.default_rng(1)
+    t = [to_torch(f32(v), DEV) for v in (rng.uniform(0, 48, (n, 2)), np.tile([0.1, 0, 0.1], (n, 1)), np.full(n, 0.5),
+                                         np.ones((n, 3)), np.ones(n))]
+    ids = torch.arange(n, dtype=torch.int32, device=DEV)
+    empty = torch.zeros(6, 2, dtype=torch.int32, device=DEV)
+    inverted = torch.tensor([[n, 0], [1, 0], [n - 1, 3], [0, 0], [7, 6], [n, n - 1]], dtype=torch.int32, device=DEV)
+    radius = torch.full((n,), 5, dtype=torch.int32, device=DEV)
+    res = []
+    for r in (empty, inverted):
+        o = tc.tcgs_render_fwd(cam, tc.render_opts("fp32"), r, ids, *t[:4], bg=(0.25, 0.5, 0.75))
+        g = tc.tcgs_render_bwd(cam, tc.render_opts("fp32"), r, ids, *t[:4], o["img"], o["T_final"], o["n_contrib"],
+                               torch.ones_like(o["img"]))
+        res.append((*o.values(), *g.values(), tc.tcgs_tile_features(cam, r, ids, t[0], t[1], t[2], t[4], radius)))
+    for a, b in zip(*res):
+        assert torch.equal(a, b)
