@@ -110,7 +110,8 @@ typedef struct {
                                 changes the schedule, never the image); NULL: one CTA per tile.  A view
                                 of at most tcgs_tc_wave_tiles() tiles is rendered one CTA per tile even
                                 when an order is given: every tile then starts in the first wave.
-                                TCGS_FP32 and tcgs_render_bwd start one CTA per tile in this order */
+                                TCGS_FP32 and tcgs_render_bwd do not read it (their orders:
+                                tcgs_render_fwd_fp32_ordered, tcgs_render_bwd_ordered) */
     uint32_t* work_counter;  /* device uint32, required with tile_order: the grid's next-tile counter,
                                 zeroed by the call */
     int32_t pixels_per_thread; /* 0 or 1: the tensor-core renderer's consumer threads blend one pixel
@@ -294,6 +295,15 @@ TCGS_API tcgs_status tcgs_render_fwd(const tcgs_camera* cam /* host */, const tc
                             const float* bg3 /* host */, float* img, float* T_final, uint32_t* n_contrib,
                             tcgs_stream stream);
 
+/* tcgs_render_fwd at TCGS_FP32 with one CTA per tile, started in the order of tile_order (device [num_tiles], a
+ * permutation of all tiles such as tcgs_tile_order's; NULL: raster order): the same outputs, and the longest tiles
+ * need not start last.  opts->precision must be TCGS_FP32. */
+TCGS_API tcgs_status tcgs_render_fwd_fp32_ordered(const tcgs_camera* cam /* host */, const tcgs_render_opts* opts /* host */,
+                            const uint32_t* tile_order, const uint32_t* tile_ranges, const uint32_t* ids_sorted,
+                            const float* mean2d, const float* conic, const float* opacity, const float* rgb,
+                            const float* bg3 /* host */, float* img, float* T_final, uint32_t* n_contrib,
+                            tcgs_stream stream);
+
 /*
  * Longest-first order of a view's tiles for the persistent renderer (tcgs_render_opts.tile_order):
  * every tile once, grouped by floor(log2(list length)) from the longest group to the empty tiles,
@@ -410,6 +420,15 @@ TCGS_API tcgs_status tcgs_sched_order(const float* cost, const uint32_t* items, 
 TCGS_API tcgs_status tcgs_render_bwd(const tcgs_camera* cam /* host */, const tcgs_render_opts* opts /* host */,
                             const uint32_t* tile_ranges, const uint32_t* ids_sorted, const float* mean2d,
                             const float* conic, const float* opacity, const float* rgb,
+                            const float* bg3 /* host */, const float* img, const float* T_final,
+                            const uint32_t* n_contrib, const float* dL_dimg, float* dmean2d, float* dconic,
+                            float* dopacity, float* drgb, tcgs_stream stream);
+
+/* tcgs_render_bwd with its CTAs, one per tile, started in the order of tile_order (device [num_tiles], a permutation
+ * of all tiles: a tile named twice adds its gradients twice; NULL: raster order). */
+TCGS_API tcgs_status tcgs_render_bwd_ordered(const tcgs_camera* cam /* host */, const tcgs_render_opts* opts /* host */,
+                            const uint32_t* tile_order, const uint32_t* tile_ranges, const uint32_t* ids_sorted,
+                            const float* mean2d, const float* conic, const float* opacity, const float* rgb,
                             const float* bg3 /* host */, const float* img, const float* T_final,
                             const uint32_t* n_contrib, const float* dL_dimg, float* dmean2d, float* dconic,
                             float* dopacity, float* drgb, tcgs_stream stream);

@@ -243,7 +243,8 @@ def tcgs_bin_sort_noalloc(cam, mean2d, radius, depth, capacity: int, out=None, s
 
 
 def tcgs_render_fwd(cam, opts, tile_ranges, ids_sorted, mean2d, conic, opacity, rgb, bg=(0.0, 0.0, 0.0), out=None,
-                    stream=None) -> dict:
+                    stream=None, fp32_order=None) -> dict:
+    """fp32_order (precision "fp32" only): the order in which the tiles start (tcgs_render_fwd_fp32_ordered)."""
     c = _cam(cam)
     if not isinstance(opts, tcgs_render_opts):
         opts = render_opts(**opts)
@@ -254,8 +255,11 @@ def tcgs_render_fwd(cam, opts, tile_ranges, ids_sorted, mean2d, conic, opacity, 
                    n_contrib=torch.empty(H, W, dtype=torch.int32, device=dev))
     bg3 = (ctypes.c_float * 3)(*[float(b) for b in bg])
     f = torch.float32
-    check("tcgs_render_fwd", _L().tcgs_render_fwd(
-        ctypes.byref(c), ctypes.byref(opts), _ptr(tile_ranges, torch.int32, "tile_ranges"),
+    fn, order = _L().tcgs_render_fwd, ()
+    if fp32_order is not None:
+        fn, order = _L().tcgs_render_fwd_fp32_ordered, (_ptr(fp32_order, torch.int32, "fp32_order"),)
+    check("tcgs_render_fwd", fn(
+        ctypes.byref(c), ctypes.byref(opts), *order, _ptr(tile_ranges, torch.int32, "tile_ranges"),
         _ptr(ids_sorted, torch.int32, "ids_sorted"), _ptr(mean2d, f, "mean2d"), _ptr(conic, f, "conic"),
         _ptr(opacity, f, "opacity"), _ptr(rgb, f, "rgb"), ctypes.cast(bg3, ctypes.c_void_p),
         _ptr(out["img"], f), _ptr(out["T_final"], f), _ptr(out["n_contrib"], torch.int32), _stream(stream)))
@@ -263,7 +267,8 @@ def tcgs_render_fwd(cam, opts, tile_ranges, ids_sorted, mean2d, conic, opacity, 
 
 
 def tcgs_render_bwd(cam, opts, tile_ranges, ids_sorted, mean2d, conic, opacity, rgb, img, T_final, n_contrib,
-                    dL_dimg, bg=(0.0, 0.0, 0.0), grads=None, stream=None) -> dict:
+                    dL_dimg, bg=(0.0, 0.0, 0.0), grads=None, stream=None, tile_order=None) -> dict:
+    """tile_order: the order in which the tiles start (tcgs_render_bwd_ordered)."""
     c = _cam(cam)
     if not isinstance(opts, tcgs_render_opts):
         opts = render_opts(**opts)
@@ -274,8 +279,9 @@ def tcgs_render_bwd(cam, opts, tile_ranges, ids_sorted, mean2d, conic, opacity, 
                          _zeros(((P, 2), dev), ((P, 3), dev), ((P,), dev), ((P, 3), dev))))
     bg3 = (ctypes.c_float * 3)(*[float(b) for b in bg])
     f = torch.float32
-    check("tcgs_render_bwd", _L().tcgs_render_bwd(
-        ctypes.byref(c), ctypes.byref(opts), _ptr(tile_ranges, torch.int32, "tile_ranges"),
+    check("tcgs_render_bwd", _L().tcgs_render_bwd_ordered(
+        ctypes.byref(c), ctypes.byref(opts), _ptr(tile_order, torch.int32, "tile_order"),
+        _ptr(tile_ranges, torch.int32, "tile_ranges"),
         _ptr(ids_sorted, torch.int32, "ids_sorted"), _ptr(mean2d, f, "mean2d"), _ptr(conic, f, "conic"),
         _ptr(opacity, f, "opacity"), _ptr(rgb, f, "rgb"), ctypes.cast(bg3, ctypes.c_void_p), _ptr(img, f, "img"),
         _ptr(T_final, f, "T_final"), _ptr(n_contrib, torch.int32, "n_contrib"), _ptr(dL_dimg, f, "dL_dimg"),
@@ -599,20 +605,23 @@ class FramePipeline:
 
 # ---------------------------------------------------------------- autograd
 
-def _training_order(cam, tile_ranges):
-    """Longest-first tile order and the renderer's counter for views of more tiles than one wave (else None):
-    the renderer then starts its longest tiles first instead of ending with them."""
-    if tile_ranges.shape[0] <= tcgs_tc_wave_tiles():
-        return None, None
-    return (tcgs_tile_order(cam, tile_ranges), torch.empty(1, dtype=torch.int32, device=tile_ranges.device))
+def _render_training(cam, precision, alpha_max, tile_ranges, ids_sorted, mean2d, conic, opacity, rgb, bg):
+    """tcgs_render_fwd with the tiles longest list first in views of more tiles than one wave, which then do not end
+    with their longest ones.  Returns its outputs and the order (None in smaller views)."""
+    order = counter = None
+    if tile_ranges.shape[0] > tcgs_tc_wave_tiles():
+        order = tcgs_tile_order(cam, tile_ranges)
+        counter = torch.empty(1, dtype=torch.int32, device=tile_ranges.device)
+    opts = render_opts(precision, alpha_max, tile_order=order, work_counter=counter)
+    out = tcgs_render_fwd(cam, opts, tile_ranges, ids_sorted, mean2d, conic, opacity, rgb, bg=bg,
+                          fp32_order=order if opts.precision == TCGS_FP32 else None)
+    return out, order
 
 
 class _Rasterize(torch.autograd.Function):
     @staticmethod
     def forward(ctx, mean2d, conic, opacity, rgb, cam, tile_ranges, ids_sorted, precision, alpha_max, bg):
-        order, counter = _training_order(cam, tile_ranges)
-        out = tcgs_render_fwd(cam, render_opts(precision, alpha_max, tile_order=order, work_counter=counter),
-                              tile_ranges, ids_sorted, mean2d, conic, opacity, rgb, bg=bg)
+        out, order = _render_training(cam, precision, alpha_max, tile_ranges, ids_sorted, mean2d, conic, opacity, rgb, bg)
         ctx.cam, ctx.alpha_max, ctx.bg = cam, alpha_max, bg
         ctx.save_for_backward(mean2d, conic, opacity, rgb, tile_ranges, ids_sorted, out["img"], out["T_final"],
                               out["n_contrib"], order)
@@ -622,8 +631,8 @@ class _Rasterize(torch.autograd.Function):
     @staticmethod
     def backward(ctx, g_img, g_T):
         mean2d, conic, opacity, rgb, ranges, ids, img, T_final, n_contrib, order = ctx.saved_tensors
-        g = tcgs_render_bwd(ctx.cam, render_opts("fp32", ctx.alpha_max, tile_order=order), ranges, ids, mean2d, conic,
-                            opacity, rgb, img, T_final, n_contrib, g_img.contiguous(), bg=ctx.bg)
+        g = tcgs_render_bwd(ctx.cam, render_opts("fp32", ctx.alpha_max), ranges, ids, mean2d, conic, opacity, rgb, img,
+                            T_final, n_contrib, g_img.contiguous(), bg=ctx.bg, tile_order=order)
         return g["dmean2d"], g["dconic"], g["dopacity"], g["drgb"], None, None, None, None, None, None
 
 
@@ -647,9 +656,7 @@ class _RenderGaussians(torch.autograd.Function):
         bins = tcgs_bin_sort(cam, pr["mean2d"], pr["radius"], pr["depth"], capacity,
                              conic=pr["conic"] if exact_tiles else None, opacity=opacity if exact_tiles else None)
         ranges, ids = bins["tile_ranges"], bins["ids_sorted"]
-        order, counter = _training_order(cam, ranges)
-        out = tcgs_render_fwd(cam, render_opts(precision, alpha_max, tile_order=order, work_counter=counter), ranges, ids,
-                              pr["mean2d"], pr["conic"], opacity, pr["rgb"], bg=bg)
+        out, _ = _render_training(cam, precision, alpha_max, ranges, ids, pr["mean2d"], pr["conic"], opacity, pr["rgb"], bg)
         ctx.cam, ctx.sh_degree, ctx.alpha_max, ctx.bg = cam, sh_degree, alpha_max, bg
         ctx.save_for_backward(means3, scales, quats, opacity, sh, pr["mean2d"], pr["conic"], pr["rgb"], pr["radius"],
                               ranges, ids, out["img"], out["T_final"], out["n_contrib"])

@@ -64,7 +64,9 @@ SIGNATURES = {
     "tcgs_bin_sort_exact": (c_int32, [P_CAM, c_int32, V, V, V, V, V, c_int64, V, c_size_t, V, V, V, V, V]),
     "tcgs_tile_order": (c_int32, [P_CAM, V, V, V]),
     "tcgs_render_fwd": (c_int32, [P_CAM, P_OPT, V, V, V, V, V, V, V, V, V, V, V]),
+    "tcgs_render_fwd_fp32_ordered": (c_int32, [P_CAM, P_OPT] + [V] * 12),
     "tcgs_render_bwd": (c_int32, [P_CAM, P_OPT, V, V, V, V, V, V, V, V, V, V, V, V, V, V, V, V]),
+    "tcgs_render_bwd_ordered": (c_int32, [P_CAM, P_OPT] + [V] * 17),
     "tcgs_render_fwd_batched": (c_int32, [c_int32, V, P_OPT, V, V, V, c_int32, V, c_int32, V]),
     "tcgs_tile_features": (c_int32, [P_CAM, V, V, V, V, V, V, V, V, V]),
     "tcgs_feature_norm": (c_int32, [V, c_int32, V, V]),

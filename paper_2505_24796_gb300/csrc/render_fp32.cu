@@ -520,10 +520,10 @@ namespace tcgs {
 tcgs_status launch_render_fp32(const tcgs_camera* cam, const tcgs_render_opts* opts, const uint32_t* tile_ranges,
                                const uint32_t* ids_sorted, const float* mean2d, const float* conic,
                                const float* opacity, const float* rgb, const float* bg3, float* img, float* T_final,
-                               uint32_t* n_contrib, cudaStream_t s) {
+                               uint32_t* n_contrib, const uint32_t* order, cudaStream_t s) {
     FwdParams p;
     p.cam = make_dev_camera(*cam);
-    p.ranges = tile_ranges; p.order = opts->tile_order; p.ids = ids_sorted; p.mean2d = mean2d; p.conic = conic; p.opacity = opacity;
+    p.ranges = tile_ranges; p.order = order; p.ids = ids_sorted; p.mean2d = mean2d; p.conic = conic; p.opacity = opacity;
     p.rgb = rgb;
     for (int i = 0; i < 3; ++i) p.bg[i] = bg3 ? bg3[i] : 0.f;
     p.alpha_max = opts->alpha_max;
@@ -544,12 +544,13 @@ tcgs_status launch_render_fp32(const tcgs_camera* cam, const tcgs_render_opts* o
 }
 }  // namespace tcgs
 
-extern "C" tcgs_status tcgs_render_bwd(const tcgs_camera* cam, const tcgs_render_opts* opts,
-                                       const uint32_t* tile_ranges, const uint32_t* ids_sorted, const float* mean2d,
-                                       const float* conic, const float* opacity, const float* rgb, const float* bg3,
-                                       const float* img, const float* T_final, const uint32_t* n_contrib,
-                                       const float* dL_dimg, float* dmean2d, float* dconic, float* dopacity,
-                                       float* drgb, tcgs_stream stream) {
+extern "C" tcgs_status tcgs_render_bwd_ordered(const tcgs_camera* cam, const tcgs_render_opts* opts,
+                                               const uint32_t* tile_order, const uint32_t* tile_ranges,
+                                               const uint32_t* ids_sorted, const float* mean2d, const float* conic,
+                                               const float* opacity, const float* rgb, const float* bg3,
+                                               const float* img, const float* T_final, const uint32_t* n_contrib,
+                                               const float* dL_dimg, float* dmean2d, float* dconic,
+                                               float* dopacity, float* drgb, tcgs_stream stream) {
     using namespace tcgs;
     if (!valid_camera(cam) || !opts || !tile_ranges || !ids_sorted || !mean2d || !conic || !opacity || !rgb ||
         !img || !T_final || !n_contrib || !dL_dimg || !dmean2d || !dconic || !dopacity || !drgb)
@@ -559,7 +560,7 @@ extern "C" tcgs_status tcgs_render_bwd(const tcgs_camera* cam, const tcgs_render
     if (reinterpret_cast<uintptr_t>(mean2d) & 7) return TCGS_ERR_INVALID;
     BwdParams p;
     p.cam = make_dev_camera(*cam);
-    p.ranges = tile_ranges; p.order = opts->tile_order; p.ids = ids_sorted; p.mean2d = mean2d; p.conic = conic; p.opacity = opacity;
+    p.ranges = tile_ranges; p.order = tile_order; p.ids = ids_sorted; p.mean2d = mean2d; p.conic = conic; p.opacity = opacity;
     p.rgb = rgb;
     for (int i = 0; i < 3; ++i) p.bg[i] = bg3 ? bg3[i] : 0.f;
     p.alpha_max = opts->alpha_max;
@@ -572,4 +573,14 @@ extern "C" tcgs_status tcgs_render_bwd(const tcgs_camera* cam, const tcgs_render
     count_launches(1);
     TCGS_CHECK_LAUNCH();
     return TCGS_OK;
+}
+
+extern "C" tcgs_status tcgs_render_bwd(const tcgs_camera* cam, const tcgs_render_opts* opts,
+                                       const uint32_t* tile_ranges, const uint32_t* ids_sorted, const float* mean2d,
+                                       const float* conic, const float* opacity, const float* rgb, const float* bg3,
+                                       const float* img, const float* T_final, const uint32_t* n_contrib,
+                                       const float* dL_dimg, float* dmean2d, float* dconic, float* dopacity,
+                                       float* drgb, tcgs_stream stream) {
+    return tcgs_render_bwd_ordered(cam, opts, nullptr, tile_ranges, ids_sorted, mean2d, conic, opacity, rgb, bg3, img,
+                                   T_final, n_contrib, dL_dimg, dmean2d, dconic, dopacity, drgb, stream);
 }

@@ -932,24 +932,32 @@ namespace tcgs {
 tcgs_status launch_render_fp32(const tcgs_camera* cam, const tcgs_render_opts* opts, const uint32_t* tile_ranges,
                                const uint32_t* ids_sorted, const float* mean2d, const float* conic,
                                const float* opacity, const float* rgb, const float* bg3, float* img, float* T_final,
-                               uint32_t* n_contrib, cudaStream_t s);
+                               uint32_t* n_contrib, const uint32_t* order, cudaStream_t s);
+namespace {
+
+bool valid_render(const tcgs_camera* cam, const tcgs_render_opts* opts, const uint32_t* tile_ranges,
+                  const uint32_t* ids_sorted, const float* mean2d, const float* conic, const float* opacity,
+                  const float* rgb, const float* img, const float* T_final, const uint32_t* n_contrib) {
+    return valid_camera(cam) && opts && tile_ranges && ids_sorted && mean2d && conic && opacity && rgb && img &&
+           T_final && n_contrib && opts->alpha_max > 0.f && opts->alpha_max <= 1.f &&
+           !(reinterpret_cast<uintptr_t>(mean2d) & 7);
 }
+
+}  // namespace
+}  // namespace tcgs
 
 extern "C" tcgs_status tcgs_render_fwd(const tcgs_camera* cam, const tcgs_render_opts* opts,
                                        const uint32_t* tile_ranges, const uint32_t* ids_sorted, const float* mean2d,
                                        const float* conic, const float* opacity, const float* rgb, const float* bg3,
                                        float* img, float* T_final, uint32_t* n_contrib, tcgs_stream stream) {
     using namespace tcgs;
-    if (!valid_camera(cam) || !opts || !tile_ranges || !ids_sorted || !mean2d || !conic || !opacity || !rgb ||
-        !img || !T_final || !n_contrib)
+    if (!valid_render(cam, opts, tile_ranges, ids_sorted, mean2d, conic, opacity, rgb, img, T_final, n_contrib))
         return TCGS_ERR_INVALID;
-    if (!(opts->alpha_max > 0.f && opts->alpha_max <= 1.f)) return TCGS_ERR_INVALID;
-    if (reinterpret_cast<uintptr_t>(mean2d) & 7) return TCGS_ERR_INVALID;
     cudaStream_t s = (cudaStream_t)stream;
     switch (opts->precision) {
         case TCGS_FP32:
             return launch_render_fp32(cam, opts, tile_ranges, ids_sorted, mean2d, conic, opacity, rgb, bg3, img,
-                                      T_final, n_contrib, s);
+                                      T_final, n_contrib, nullptr, s);
         case TCGS_TC_FP16:
         case TCGS_TC_FP16_SPLIT:
         case TCGS_TC_FP8:
@@ -962,6 +970,20 @@ extern "C" tcgs_status tcgs_render_fwd(const tcgs_camera* cam, const tcgs_render
         default:
             return TCGS_ERR_INVALID;
     }
+}
+
+extern "C" tcgs_status tcgs_render_fwd_fp32_ordered(const tcgs_camera* cam, const tcgs_render_opts* opts,
+                                                    const uint32_t* tile_order, const uint32_t* tile_ranges,
+                                                    const uint32_t* ids_sorted, const float* mean2d,
+                                                    const float* conic, const float* opacity, const float* rgb,
+                                                    const float* bg3, float* img, float* T_final,
+                                                    uint32_t* n_contrib, tcgs_stream stream) {
+    using namespace tcgs;
+    if (!valid_render(cam, opts, tile_ranges, ids_sorted, mean2d, conic, opacity, rgb, img, T_final, n_contrib) ||
+        opts->precision != TCGS_FP32)
+        return TCGS_ERR_INVALID;
+    return launch_render_fp32(cam, opts, tile_ranges, ids_sorted, mean2d, conic, opacity, rgb, bg3, img, T_final,
+                              n_contrib, tile_order, (cudaStream_t)stream);
 }
 
 extern "C" tcgs_status tcgs_render_fwd_batched(int32_t n_views, const tcgs_view* views, const tcgs_render_opts* opts,

@@ -165,3 +165,35 @@ def test_inverted_ranges_are_empty_lists(tc):
         res.append((*o.values(), *g.values(), tc.tcgs_tile_features(cam, r, ids, t[0], t[1], t[2], t[4], radius)))
     for a, b in zip(*res):
         assert torch.equal(a, b)
+
+
+def test_fp32_paths_take_their_order_from_their_own_entry_points(tc):
+    """The tensor-core renderer's order in the options, here one that names a tile twice and leaves one out, is not
+    read by TCGS_FP32 and the backward; a permutation given to their ordered entry points changes neither image
+    nor gradients (a Gaussian lies in one tile here, so that its sums do not depend on the tiles' order)."""
+    cam = scenes.pinhole(64, 48, fx=50.0)
+    rng = np.random.default_rng(4)
+    n, nt = 240, 12
+    tile = np.arange(n) // 20
+    t = [to_torch(f32(v), DEV) for v in (np.stack([tile % 4 * 16, tile // 4 * 16], 1) + rng.uniform(0, 16, (n, 2)),
+                                         np.tile([0.05, 0.01, 0.05], (n, 1)), rng.uniform(0.1, 0.6, n), rng.uniform(0, 1, (n, 3)))]
+    ids = torch.arange(n, dtype=torch.int32, device=DEV)
+    ranges = torch.stack([torch.arange(nt) * 20, torch.arange(1, nt + 1) * 20], 1).int().to(DEV)
+    bad = torch.arange(nt, dtype=torch.int32, device=DEV)
+    bad[3] = 5
+    perm = torch.arange(nt - 1, -1, -1, dtype=torch.int32, device=DEV)
+    counter = torch.zeros(1, dtype=torch.int32, device=DEV)
+    dl = torch.randn(3, 48, 64, device=DEV)
+    res = []
+    for opts, order in ((tc.render_opts("fp32"), None), (tc.render_opts("fp32", tile_order=bad, work_counter=counter), None),
+                        (tc.render_opts("fp32"), perm)):
+        kw = ({}, {}) if order is None else (dict(fp32_order=order), dict(tile_order=order))
+        o = dict(img=torch.full((3, 48, 64), -1.0, device=DEV), T_final=torch.full((48, 64), -1.0, device=DEV),
+                 n_contrib=torch.full((48, 64), -1, dtype=torch.int32, device=DEV))
+        tc.tcgs_render_fwd(cam, opts, ranges, ids, *t, out=o, **kw[0])
+        g = tc.tcgs_render_bwd(cam, opts, ranges, ids, *t, o["img"], o["T_final"], o["n_contrib"], dl, **kw[1])
+        res.append((*o.values(), *g.values()))
+        for a, b in zip(res[0], res[-1]):
+            assert torch.equal(a, b)
+    with pytest.raises(tc.TcgsError):
+        tc.tcgs_render_fwd(cam, tc.render_opts("tc_fp16_split"), ranges, ids, *t, fp32_order=perm)
