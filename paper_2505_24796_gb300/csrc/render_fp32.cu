@@ -1,5 +1,7 @@
 // render_fp32.cu -- conditional alpha-blending on CUDA cores (Algorithm 1, Eq. 4-6): the FP32 forward
 // and the backward replay.
+#include <type_traits>
+
 #include "common.cuh"
 #include "pairs.cuh"
 
@@ -295,7 +297,8 @@ __global__ void __launch_bounds__(kBwdThreads, 4) k_render_bwd(BwdParams p) {
     const PairPixels q = pair_pixels(warp, lane);
     const float cx = (float)(tx * kTile + kTile / 2), cy = (float)(ty * kTile + kTile / 2);
     const uint32_t start = p.ranges[2 * tile], stop = p.ranges[2 * tile + 1];
-    const uint32_t end = stop > start ? stop : start;   // an inverted range is an empty list
+    if (stop <= start) return;   // an empty list (an inverted range is one): no gradient
+    const uint32_t end = stop;
     const float amax = p.alpha_max, inf = __int_as_float(0x7f800000);
 
     // per pixel: n_contrib, -dL/dimg, T_final, the colour still to come, the replayed T
@@ -384,111 +387,117 @@ __global__ void __launch_bounds__(kBwdThreads, 4) k_render_bwd(BwdParams p) {
         }
         if (lane < kBwdGroup) s_list[warp][n + lane] = (uint8_t)kBwdBatch;   // pads the last group
         __syncwarp();
-        for (uint32_t at = 0; at < n; at += kBwdGroup) {
-            const uint32_t four = *reinterpret_cast<const uint32_t*>(&s_list[warp][at]);
-            // alphas of the four fragments (negated; 0: the pixel does not blend it), exp(power) (0: or with a
-            // clamped alpha), dx, dy
-            f32x2 na[kBwdGroup], G[kBwdGroup], dx[kBwdGroup], dy[kBwdGroup];
-            bool any = false;
+        // two copies of the replay: the masks that odd values need cost 5% in one (1024 x 512, 250k Gaussians: 307 and
+        // 278 us)
+        auto replay = [&](auto odd_values) {
+            constexpr bool kStrict = decltype(odd_values)::value;
+            for (uint32_t at = 0; at < n; at += kBwdGroup) {
+                const uint32_t four = *reinterpret_cast<const uint32_t*>(&s_list[warp][at]);
+                // alphas of the four fragments (negated; 0: the pixel does not blend it), exp(power) (0: or with a
+                // clamped alpha), dx, dy
+                f32x2 na[kBwdGroup], G[kBwdGroup], dx[kBwdGroup], dy[kBwdGroup];
+                bool any = false;
 #pragma unroll
-            for (int f = 0; f < kBwdGroup; ++f) {
-                const uint32_t j = (four >> (8 * f)) & 0xFFu;
-                const PairRec& r = s_f[j];
-                const ulonglong2 xa = r.q[0], bc = r.q[1], yo = r.q[2];
-                dx[f] = add2(xa.x, npx);
-                dy[f] = add2(yo.x, npy);
-                const f32x2 pw = pair_power(xa.y, bc.x, bc.y, dx[f], dy[f]);
-                const float G0 = expf(lo2(pw)), G1 = expf(hi2(pw));
-                const f32x2 raw = mul2(yo.y, pack2f(G0, G1));   // -o exp(power)
-                const float a0 = fmaxf(-amax, lo2(raw)), a1 = fmaxf(-amax, hi2(raw));
-                bool in0 = a0 <= -kCullAlpha && b0 + j < nc[0], in1 = a1 <= -kCullAlpha && b0 + j < nc[1];
-                if (kEarly) {   // the forward's test
-                    const float lno = r.lno();
-                    in0 = in0 && !(lo2(pw) + lno < kBetaCull);
-                    in1 = in1 && !(hi2(pw) + lno < kBetaCull);
+                for (int f = 0; f < kBwdGroup; ++f) {
+                    const uint32_t j = (four >> (8 * f)) & 0xFFu;
+                    const PairRec& r = s_f[j];
+                    const ulonglong2 xa = r.q[0], bc = r.q[1], yo = r.q[2];
+                    dx[f] = add2(xa.x, npx);
+                    dy[f] = add2(yo.x, npy);
+                    const f32x2 pw = pair_power(xa.y, bc.x, bc.y, dx[f], dy[f]);
+                    const float G0 = expf(lo2(pw)), G1 = expf(hi2(pw));
+                    const f32x2 raw = mul2(yo.y, pack2f(G0, G1));   // -o exp(power)
+                    const float a0 = fmaxf(-amax, lo2(raw)), a1 = fmaxf(-amax, hi2(raw));
+                    bool in0 = a0 <= -kCullAlpha && b0 + j < nc[0], in1 = a1 <= -kCullAlpha && b0 + j < nc[1];
+                    if (kEarly) {   // the forward's test
+                        const float lno = r.lno();
+                        in0 = in0 && !(lo2(pw) + lno < kBetaCull);
+                        in1 = in1 && !(hi2(pw) + lno < kBetaCull);
+                    }
+                    any = any || in0 || in1;
+                    na[f] = pack2f(in0 ? a0 : 0.f, in1 ? a1 : 0.f);
+                    G[f] = pack2f(in0 && lo2(raw) >= -amax ? G0 : 0.f, in1 && hi2(raw) >= -amax ? G1 : 0.f);
                 }
-                any = any || in0 || in1;
-                na[f] = pack2f(in0 ? a0 : 0.f, in1 ? a1 : 0.f);
-                G[f] = pack2f(in0 && lo2(raw) >= -amax ? G0 : 0.f, in1 && hi2(raw) >= -amax ? G1 : 0.f);
-            }
-            const bool u16 = lane & 16, u8 = lane & 8, u4 = lane & 4, u2 = lane & 2, u1 = lane & 1;
-            const uint32_t jl = (four >> ((u16 ? 8 : 0) + (u8 ? 16 : 0))) & 0xFFu;   // this quarter's fragment
-            float* part = s_part[warp][jl];
-            if (!__any_sync(0xffffffffu, any)) {
-                part[lane & 7] = 0.f;
-                part[8] = 0.f;
-                continue;
-            }
-            float z[2][kBwdParams];
-#pragma unroll
-            for (int f = 0; f < kBwdGroup; f += 2) {
-                float v[2][kBwdParams];
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const f32x2 na_f = na[f + e], G_f = G[f + e];
-                    f32x2 dx_f = dx[f + e], dy_f = dy[f + e];
-                    const PairRec& r = s_f[(four >> (8 * (f + e))) & 0xFFu];
-                    f32x2 cr = r.q[3].x, cg = r.q[3].y, cb = r.q[4].x, h0 = ng0, h1 = ng1, h2 = ng2;
-                    if (strict) {   // 0 times an infinity or a NaN would reach what does not blend it
-                        cr = where2(na_f, cr); cg = where2(na_f, cg); cb = where2(na_f, cb);
-                        h0 = where2(na_f, h0); h1 = where2(na_f, h1); h2 = where2(na_f, h2);
-                    }
-                    const f32x2 wn = mul2(na_f, T);   // -alpha T
-                    R0 = fma2(cr, wn, R0);
-                    R1 = fma2(cg, wn, R1);
-                    R2 = fma2(cb, wn, R2);
-                    // -1 / (1 - alpha): the approximate reciprocal and one Newton-Raphson step (the
-                    // correctly rounded value for every float in (6e-8, 1], by exhaustive comparison)
-                    const f32x2 om = add2(one, na_f);
-                    const f32x2 r0 = pack2f(rcp_approx(-lo2(om)), rcp_approx(-hi2(om)));
-                    const f32x2 nia = fma2(fma2(om, r0, one), r0, r0);
-                    f32x2 X0 = R0, X1 = R1, X2 = R2;
-                    if (has_bg) {
-                        X0 = fma2(Tf, pack2f(bg0, bg0), R0);
-                        X1 = fma2(Tf, pack2f(bg1, bg1), R1);
-                        X2 = fma2(Tf, pack2f(bg2, bg2), R2);
-                    }
-                    // -dL/dalpha = -g (c T - (R + T_final bg) / (1 - alpha))
-                    const f32x2 A0 = fma2(cr, T, mul2(X0, nia)), A1 = fma2(cg, T, mul2(X1, nia)), A2 = fma2(cb, T, mul2(X2, nia));
-                    const f32x2 nd_all = fma2(h2, A2, fma2(h0, A0, mul2(h1, A1)));
-                    const f32x2 nd = where2(G_f, nd_all);
-                    const f32x2 d = mul2(nd, na_f);   // dL/dpower
-                    const f32x2 bx = mul2(r.q[1].x, dx_f), cy = mul2(r.q[1].y, dy_f);
-                    f32x2 m0 = fma2(r.q[1].x, dy_f, mul2(r.q[0].y, dx_f));   // -(a dx + b dy)
-                    f32x2 m1 = pack2f(__fadd_rn(lo2(bx), lo2(cy)), __fadd_rn(hi2(bx), hi2(cy)));   // -(b dx + c dy)
-                    if (strict) {   // nor may the geometry's, where d is 0
-                        m0 = where2(G_f, m0); m1 = where2(G_f, m1);
-                        dx_f = where2(G_f, dx_f); dy_f = where2(G_f, dy_f);
-                    }
-                    const f32x2 ddx = mul2(d, dx_f), ddy = mul2(d, dy_f);
-                    v[e][0] = dot2(d, m0);
-                    v[e][1] = dot2(d, m1);
-                    v[e][2] = dot2(ddx, dx_f);
-                    v[e][3] = dot2(ddx, dy_f);
-                    v[e][4] = dot2(ddy, dy_f);
-                    v[e][5] = dot2(nd, G_f);
-                    v[e][6] = dot2(wn, h0);
-                    v[e][7] = dot2(wn, h1);
-                    v[e][8] = dot2(wn, h2);
-                    T = fma2(na_f, T, T);
+                const bool u16 = lane & 16, u8 = lane & 8, u4 = lane & 4, u2 = lane & 2, u1 = lane & 1;
+                const uint32_t jl = (four >> ((u16 ? 8 : 0) + (u8 ? 16 : 0))) & 0xFFu;   // this quarter's fragment
+                float* part = s_part[warp][jl];
+                if (!__any_sync(0xffffffffu, any)) {
+                    part[lane & 7] = 0.f;
+                    part[8] = 0.f;
+                    continue;
                 }
+                float z[2][kBwdParams];
 #pragma unroll
-                for (int k = 0; k < kBwdParams; ++k) z[f / 2][k] = exchange(v[0][k], v[1][k], u16, 16);
+                for (int f = 0; f < kBwdGroup; f += 2) {
+                    float v[2][kBwdParams];
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const f32x2 na_f = na[f + e], G_f = G[f + e];
+                        f32x2 dx_f = dx[f + e], dy_f = dy[f + e];
+                        const PairRec& r = s_f[(four >> (8 * (f + e))) & 0xFFu];
+                        f32x2 cr = r.q[3].x, cg = r.q[3].y, cb = r.q[4].x, h0 = ng0, h1 = ng1, h2 = ng2;
+                        if (kStrict) {   // 0 times an infinity or a NaN would reach what does not blend it
+                            cr = where2(na_f, cr); cg = where2(na_f, cg); cb = where2(na_f, cb);
+                            h0 = where2(na_f, h0); h1 = where2(na_f, h1); h2 = where2(na_f, h2);
+                        }
+                        const f32x2 wn = mul2(na_f, T);   // -alpha T
+                        R0 = fma2(cr, wn, R0);
+                        R1 = fma2(cg, wn, R1);
+                        R2 = fma2(cb, wn, R2);
+                        // -1 / (1 - alpha): the approximate reciprocal and one Newton-Raphson step (the
+                        // correctly rounded value for every float in (6e-8, 1], by exhaustive comparison)
+                        const f32x2 om = add2(one, na_f);
+                        const f32x2 r0 = pack2f(rcp_approx(-lo2(om)), rcp_approx(-hi2(om)));
+                        const f32x2 nia = fma2(fma2(om, r0, one), r0, r0);
+                        f32x2 X0 = R0, X1 = R1, X2 = R2;
+                        if (has_bg) {
+                            X0 = fma2(Tf, pack2f(bg0, bg0), R0);
+                            X1 = fma2(Tf, pack2f(bg1, bg1), R1);
+                            X2 = fma2(Tf, pack2f(bg2, bg2), R2);
+                        }
+                        // -dL/dalpha = -g (c T - (R + T_final bg) / (1 - alpha))
+                        const f32x2 A0 = fma2(cr, T, mul2(X0, nia)), A1 = fma2(cg, T, mul2(X1, nia)), A2 = fma2(cb, T, mul2(X2, nia));
+                        const f32x2 nd_all = fma2(h2, A2, fma2(h0, A0, mul2(h1, A1)));
+                        const f32x2 nd = where2(G_f, nd_all);
+                        const f32x2 d = mul2(nd, na_f);   // dL/dpower
+                        const f32x2 bx = mul2(r.q[1].x, dx_f), cy = mul2(r.q[1].y, dy_f);
+                        f32x2 m0 = fma2(r.q[1].x, dy_f, mul2(r.q[0].y, dx_f));   // -(a dx + b dy)
+                        f32x2 m1 = pack2f(__fadd_rn(lo2(bx), lo2(cy)), __fadd_rn(hi2(bx), hi2(cy)));   // -(b dx + c dy)
+                        if (kStrict) {   // nor may the geometry's, where d is 0
+                            m0 = where2(G_f, m0); m1 = where2(G_f, m1);
+                            dx_f = where2(G_f, dx_f); dy_f = where2(G_f, dy_f);
+                        }
+                        const f32x2 ddx = mul2(d, dx_f), ddy = mul2(d, dy_f);
+                        v[e][0] = dot2(d, m0);
+                        v[e][1] = dot2(d, m1);
+                        v[e][2] = dot2(ddx, dx_f);
+                        v[e][3] = dot2(ddx, dy_f);
+                        v[e][4] = dot2(ddy, dy_f);
+                        v[e][5] = dot2(nd, G_f);
+                        v[e][6] = dot2(wn, h0);
+                        v[e][7] = dot2(wn, h1);
+                        v[e][8] = dot2(wn, h2);
+                        T = fma2(na_f, T, T);
+                    }
+#pragma unroll
+                    for (int k = 0; k < kBwdParams; ++k) z[f / 2][k] = exchange(v[0][k], v[1][k], u16, 16);
+                }
+                float y[kBwdParams];
+#pragma unroll
+                for (int k = 0; k < kBwdParams; ++k) y[k] = exchange(z[0][k], z[1][k], u8, 8);
+                // value 4 bit2 + 2 bit1 + bit0 of the first eight ends in each lane of the quarter, the ninth in all
+                const float e0 = exchange(y[0], y[4], u4, 4), e1 = exchange(y[1], y[5], u4, 4);
+                const float e2 = exchange(y[2], y[6], u4, 4), e3 = exchange(y[3], y[7], u4, 4);
+                const float k0 = exchange(e0, e2, u2, 2), k1 = exchange(e1, e3, u2, 2);
+                const float mine = exchange(k0, k1, u1, 1);
+                float ninth = y[8];
+#pragma unroll
+                for (int o = 4; o > 0; o >>= 1) ninth += __shfl_xor_sync(0xffffffffu, ninth, o);
+                part[lane & 7] = mine;
+                if ((lane & 7) == 0) part[8] = ninth;
             }
-            float y[kBwdParams];
-#pragma unroll
-            for (int k = 0; k < kBwdParams; ++k) y[k] = exchange(z[0][k], z[1][k], u8, 8);
-            // value 4 bit2 + 2 bit1 + bit0 of the first eight ends in each lane of the quarter, the ninth in all
-            const float e0 = exchange(y[0], y[4], u4, 4), e1 = exchange(y[1], y[5], u4, 4);
-            const float e2 = exchange(y[2], y[6], u4, 4), e3 = exchange(y[3], y[7], u4, 4);
-            const float k0 = exchange(e0, e2, u2, 2), k1 = exchange(e1, e3, u2, 2);
-            const float mine = exchange(k0, k1, u1, 1);
-            float ninth = y[8];
-#pragma unroll
-            for (int o = 4; o > 0; o >>= 1) ninth += __shfl_xor_sync(0xffffffffu, ninth, o);
-            part[lane & 7] = mine;
-            if ((lane & 7) == 0) part[8] = ninth;
-        }
+        };
+        if (strict) replay(std::true_type{}); else replay(std::false_type{});
         __syncthreads();
         // thread t adds the warps' sums of fragment t
         float s[kBwdParams] = {};
