@@ -7,7 +7,7 @@
 // queue is ordered longest-predicted first.  Its training data are the per-tile costs the
 // renderer itself records (tile_stats).
 //
-// Kernels: per-tile features (one block per tile), feature normaliser, MLP forward, MLP backward
+// Kernels: per-tile features, feature normaliser, MLP forward, MLP backward
 // (mean squared error), Adam.  The ordering sort lives with the radix sort in binsort.cu.
 #include <mutex>
 
@@ -28,13 +28,17 @@ __device__ __forceinline__ float h16(float x) { return __half2float(__float2half
 // ---------------------------------------------------------------- features
 
 constexpr int kFewTilesPerSm = 4;
+constexpr int kWarpTiles = 8;   // tiles a block where each has a warp
 
-// One block of NT threads per tile.  Bound by the latency of two dependent gathers (id, then the
-// Gaussian's values from L2) on lists of thousands of entries, so a tile gets as many threads as keep
-// enough of them in flight: 16 views of 320 x 240 (300 tiles each, about 8000 entries a tile) took 8.13 ms
-// with one warp a tile and take 0.75 ms, bound by the gathers' requests (seven a list entry, 32 lines each).
-template <int NT, bool kPairs>
-__global__ void __launch_bounds__(NT) k_tile_features(DevCamera cam, const uint32_t* __restrict__ ranges,
+// NT threads per tile, kTiles tiles a block (several only with a warp each).  Bound by the latency of two dependent
+// gathers (id, then the Gaussian's values from L2), so a thread has kDeep entries in flight, and where the view has few
+// tiles a tile gets many threads: 16 views of 320 x 240 (300 tiles each, about 8000 entries a tile) took 8.13 ms
+// with one warp a tile and one entry in flight and take 0.75 ms, bound by the gathers' requests (seven a list
+// entry, 32 lines each).  Where the tiles' warps fill the chip, a warp each is faster than a block of 128
+// (3840 x 2160, 1M small footprints: 69 and 159 us; 1920 x 1080, 300k wide ones: 496 and 648 us): nothing waits on
+// barriers, and the lists that neighbouring tiles share are walked at the same time.
+template <int NT, int kTiles, bool kPairs>
+__global__ void __launch_bounds__(NT * kTiles) k_tile_features(DevCamera cam, const uint32_t* __restrict__ ranges,
                                                       const uint32_t* __restrict__ ids,
                                                       const float* __restrict__ mean2d,
                                                       const float* __restrict__ conic,
@@ -43,14 +47,15 @@ __global__ void __launch_bounds__(NT) k_tile_features(DevCamera cam, const uint3
                                                       const int32_t* __restrict__ radius, float* __restrict__ feat) {
     constexpr int kSums = 6, kDeep = 4;   // entries a thread has in flight
     __shared__ float s_sum[NT / 32][kSums];
-    const int tile = blockIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int tile = kTiles == 1 ? blockIdx.x : blockIdx.x * kTiles + warp, tid = kTiles == 1 ? threadIdx.x : lane;
+    if (kTiles > 1 && tile >= cam.grid_w * cam.grid_h) return;
     const int tx = tile % cam.grid_w, ty = tile / cam.grid_w;
     const float x0 = (float)(kTile * tx), y0 = (float)(kTile * ty);
     const uint32_t start = ranges[2 * tile], end = ranges[2 * tile + 1];
     const uint32_t len = end > start ? end - start : 0u;   // an inverted range is an empty list
     float so = 0.f, mo = 0.f, dmin = 3.0e38f, dmax = -3.0e38f, sdet = 0.f, cov = 0.f;
-    for (uint32_t k0 = threadIdx.x; k0 < len; k0 += kDeep * NT) {
+    for (uint32_t k0 = tid; k0 < len; k0 += kDeep * NT) {
         uint32_t g[kDeep];
         bool in[kDeep];
 #pragma unroll
@@ -103,21 +108,23 @@ __global__ void __launch_bounds__(NT) k_tile_features(DevCamera cam, const uint3
         }
     };
     over_warp();
-    if (lane == 0) {
-        const float v[kSums] = {so, mo, dmin, dmax, sdet, cov};
+    if (NT > 32) {
+        if (lane == 0) {
+            const float v[kSums] = {so, mo, dmin, dmax, sdet, cov};
 #pragma unroll
-        for (int k = 0; k < kSums; ++k) s_sum[warp][k] = v[k];
+            for (int k = 0; k < kSums; ++k) s_sum[warp][k] = v[k];
+        }
+        __syncthreads();
+        if (warp > 0) return;
+        const bool in = lane < NT / 32;
+        so = in ? s_sum[lane][0] : 0.f;
+        mo = in ? s_sum[lane][1] : 0.f;
+        dmin = in ? s_sum[lane][2] : 3.0e38f;
+        dmax = in ? s_sum[lane][3] : -3.0e38f;
+        sdet = in ? s_sum[lane][4] : 0.f;
+        cov = in ? s_sum[lane][5] : 0.f;
+        over_warp();
     }
-    __syncthreads();
-    if (warp > 0) return;
-    const bool in = lane < NT / 32;
-    so = in ? s_sum[lane][0] : 0.f;
-    mo = in ? s_sum[lane][1] : 0.f;
-    dmin = in ? s_sum[lane][2] : 3.0e38f;
-    dmax = in ? s_sum[lane][3] : -3.0e38f;
-    sdet = in ? s_sum[lane][4] : 0.f;
-    cov = in ? s_sum[lane][5] : 0.f;
-    over_warp();
     if (lane == 0) {
         const float n = (float)len;
         const float inv = n > 0.f ? 1.f / n : 0.f;
@@ -410,12 +417,16 @@ extern "C" tcgs_status tcgs_tile_features(const tcgs_camera* cam, const uint32_t
     DeviceInfo d;
     const int sms = current_device_info(&d) ? d.sms : 128;
     const bool pairs = (reinterpret_cast<uintptr_t>(conic) & 7) == 0;
-    auto launch = [&](auto kern, int threads) {
-        kern<<<tiles, threads, 0, (cudaStream_t)stream>>>(dc, tile_ranges, ids_sorted, mean2d, conic, opacity, depth, radius,
-                                                          features);
+    auto launch = [&](auto kern, int threads, int per_block) {
+        const int blocks = tiles / per_block + (tiles % per_block != 0);
+        kern<<<blocks, threads, 0, (cudaStream_t)stream>>>(dc, tile_ranges, ids_sorted, mean2d, conic, opacity, depth, radius,
+                                                           features);
     };
-    if (tiles <= kFewTilesPerSm * sms) pairs ? launch(k_tile_features<512, true>, 512) : launch(k_tile_features<512, false>, 512);
-    else pairs ? launch(k_tile_features<128, true>, 128) : launch(k_tile_features<128, false>, 128);
+    if (tiles <= kFewTilesPerSm * sms)
+        pairs ? launch(k_tile_features<512, 1, true>, 512, 1) : launch(k_tile_features<512, 1, false>, 512, 1);
+    else
+        pairs ? launch(k_tile_features<32, kWarpTiles, true>, 32 * kWarpTiles, kWarpTiles)
+              : launch(k_tile_features<32, kWarpTiles, false>, 32 * kWarpTiles, kWarpTiles);
     count_launches(1);
     TCGS_CHECK_LAUNCH();
     return TCGS_OK;
