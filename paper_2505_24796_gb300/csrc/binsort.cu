@@ -821,8 +821,6 @@ struct SmallSortSmem {
 // warp by warp_peers and placed after the same digit's items of the lower warps and of the
 // earlier rounds.  keys_in and keys_out are distinct buffers; the CTA's last barrier makes the output
 // visible to all its threads.
-// No __restrict__: the depth kernel reads in one pass what its own threads wrote in the previous one,
-// so these loads must not take the read-only path.
 __device__ void cta_radix_pass(SmallSortSmem& sm, const uint32_t* kin, const uint32_t* vin, uint32_t* kout,
                                uint32_t* vout, uint32_t n, int shift, uint32_t mask) {
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
@@ -1159,7 +1157,7 @@ tcgs_status bin_sort(const tcgs_camera* cam, int32_t P, const float* mean2d, con
     // 3. duplication into the buffer the first tile pass reads
     int tile_bits = 0;
     while ((1 << tile_bits) < num_tiles) ++tile_bits;
-    int tpasses = tile_bits <= 8 ? 1 : (tile_bits <= 16 ? 2 : 3);
+    const int tpasses = tile_bits <= 16 ? 2 : 3;   // at least 257 tiles come here: more than 256 columns or rows
     // Two tile passes with the high tile bits and the Gaussian id in one word: the first pass writes
     // (tile >> 8, id) packed, the second sorts those words alone, writes the ids and, from per-tile
     // counts, the ranges (a third of the splat traffic and the ranges pass saved), for capacities of

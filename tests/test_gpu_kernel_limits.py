@@ -197,3 +197,33 @@ def test_fp32_paths_take_their_order_from_their_own_entry_points(tc):
             assert torch.equal(a, b)
     with pytest.raises(tc.TcgsError):
         tc.tcgs_render_fwd(cam, tc.render_opts("tc_fp16_split"), ranges, ids, *t, fp32_order=perm)
+
+
+@pytest.mark.parametrize("exact", [False, True])
+def test_packed_tile_sort_of_wide_views(tc, exact):
+    """A view of 257 x 40 tiles is sorted by radix passes: as key-value pairs below a capacity of 2^23 splats, from
+    there on as packed (tile >> 8, id) words.  The same lists and ranges either way, the oracle's for rectangles, and
+    in the common columns those of a view of 256 columns (row lists)."""
+    rng = np.random.default_rng(6)
+    P, H = 30_000, 640
+    sigma = np.exp(rng.uniform(np.log(1), np.log(25), P))
+    mean2d = f32(np.stack([rng.uniform(-30, 4140, P), rng.uniform(-30, H + 30, P)], 1))
+    radius = np.where(rng.random(P) < 0.1, 0, np.ceil(3 * sigma)).astype(np.int32)
+    depth = f32(rng.integers(1, 2000, P))
+    conic = f32(np.stack([1 / sigma ** 2, 0.5 / sigma ** 2 * rng.uniform(-1, 1, P), 1 / sigma ** 2], 1))
+    cams = {gw: scenes.pinhole(16 * gw, H, fx=500.0) for gw in (256, 257)}
+    b = oracle.bin_sort(cams[257], mean2d, radius, depth)
+    t = [to_torch(v, DEV) for v in (mean2d, radius, depth)]
+    kw = dict(conic=to_torch(conic, DEV), opacity=to_torch(f32(rng.uniform(0.003, 1, P)), DEV)) if exact else {}
+    assert b["n"] + 17 < 32 * P < 1 << 23
+    res = [tc.tcgs_bin_sort(cams[gw], *t, cap, **kw) for gw, cap in ((257, b["n"] + 17), (257, 1 << 23), (256, b["n"] + 17))]
+    assert [int(o["status"].item()) for o in res] == [0, 0, 0]
+    n = int(res[0]["n_splats"].item())
+    assert n == int(res[1]["n_splats"].item()) and (n < b["n"] if exact else n == b["n"])
+    assert torch.equal(res[0]["ids_sorted"][:n], res[1]["ids_sorted"][:n])
+    assert torch.equal(res[0]["tile_ranges"], res[1]["tile_ranges"])
+    if not exact:
+        np.testing.assert_array_equal(res[1]["ids_sorted"].cpu().numpy()[:n], b["ids"])
+        np.testing.assert_array_equal(res[1]["tile_ranges"].cpu().numpy(), b["ranges"])
+    for x, y in zip(_lists(res[1], 257, 256), _lists(res[2], 256, 256)):
+        assert torch.equal(x, y)
