@@ -83,7 +83,8 @@ def parse():
                          "times per frame (no headline line)")
     ap.add_argument("--render-arms", action="store_true",
                     help="profiling run: the headline frame binned once, then rendered twice by each renderer arm "
-                         "(TC split, the same kernel with the product on CUDA cores, the 3DGS-style FP32 kernel); "
+                         "(TC split, the same kernel with the product on CUDA cores, the FP32 kernel without and "
+                         "with its block tests); "
                          "render times per arm (no headline line)")
     ap.add_argument("--arms-workload", default="precision", choices=["precision", "differentiation"],
                     help="workload of --render-arms")
@@ -274,10 +275,10 @@ def bench_plain(dev, flush, stream, steps=50, warmup=5):
     r.stats = None
     out = {"workload": "plain: 128x128, fx=fy=128, 1,000 Gaussians, SH0; exact tile coverage",
            "splats": int(r.bins["n_splats"].item()), "alpha_evals": st[0] + st[1]}
-    for prec in ("tc_fp16_split", "fp32", "fp32_frag2mat"):
-        tot, stg = time_frames(r, d, prec, steps, warmup, True, flush, stream)
+    for arm, (prec, kw) in ARMS.items():
+        tot, stg = time_frames(r, d, prec, steps, warmup, True, flush, stream, **kw)
         ms = statistics.median(tot)
-        out[prec] = {"frames_per_s": 1000.0 / ms, "frame_ms": ms,
+        out[arm] = {"frames_per_s": 1000.0 / ms, "frame_ms": ms,
                      "stages_ms": dict(zip(["project", "bin_sort", "render_fwd"],
                                            [statistics.median(x) for x in stg]))}
     out["speedup_frame"] = out["fp32"]["frame_ms"] / out["tc_fp16_split"]["frame_ms"]
@@ -290,6 +291,12 @@ def bench_plain(dev, flush, stream, steps=50, warmup=5):
     diff = (r.out["img"] - img32).abs().max().item()
     out["max_abs_tc_vs_fp32"] = diff
     return out
+
+
+# Renderer arms: label -> (precision, render options).  "fp32" is the 3DGS baseline, which evaluates every list entry at
+# every pixel; with its block tests (tile_cull, the default) the same kernel skips what no pixel of a block can blend.
+ARMS = {"tc_fp16_split": ("tc_fp16_split", {}), "fp32": ("fp32", {"tile_cull": False}),
+        "fp32_block_marks": ("fp32", {"tile_cull": True}), "fp32_frag2mat": ("fp32_frag2mat", {})}
 
 
 def bench_differentiation(dev, flush):
@@ -320,7 +327,8 @@ def bench_differentiation(dev, flush):
         tc.tcgs_render_bwd(r.cam, opts, r.bins["tile_ranges"], r.bins["ids_sorted"], r.proj["mean2d"], r.proj["conic"],
                            d["opacity"], r.proj["rgb"], r.out["img"], r.out["T_final"], r.out["n_contrib"], gimg,
                            grads=grads)
-    fwd32 = _events_ms(lambda: r.render(d["opacity"], "fp32"), 10, 3, flush)
+    fwd32 = _events_ms(lambda: r.render(d["opacity"], "fp32", tile_cull=False), 10, 3, flush)
+    fwd32m = _events_ms(lambda: r.render(d["opacity"], "fp32"), 10, 3, flush)
     fwdtc = _events_ms(lambda: r.render(d["opacity"], "tc_fp16_split"), 10, 3, flush)
     fwdcc = _events_ms(lambda: r.render(d["opacity"], "fp32_frag2mat"), 10, 3, flush)
     one = _one_pixel_a_thread(r, d, flush, 10, 3)
@@ -338,13 +346,15 @@ def bench_differentiation(dev, flush):
             "splats": n_exact, "square_coverage": square,
             "alpha_evals": st[0] + st[1], "f_blend": st[0],
             "ms": {"project": proj_ms, "bin_sort": bin_ms, "render_fwd_fp32": fwd32,
+                   "render_fwd_fp32_block_marks": fwd32m,
                    "render_fwd_tc": fwdtc, "render_fwd_fp32_same_skip": fwdcc, "render_bwd": bwd_ms,
                    "project_bwd": pbwd_ms},
             "pixels_per_thread": r.pixels_per_thread, "render_fwd_one_pixel_a_thread_ms": one,
             "speedup_render": {"vs_fp32": fwd32 / fwdtc, "vs_fp32_same_skip": fwdcc / fwdtc},
             "frames_per_s_fwd": {"tc_fp16_split": 1000.0 / (proj_ms + bin_ms + fwdtc),
-                                 "fp32": 1000.0 / (proj_ms + bin_ms + fwd32)},
-            "train_step_ms_fp32": proj_ms + bin_ms + fwd32 + bwd_ms + pbwd_ms,
+                                 "fp32": 1000.0 / (proj_ms + bin_ms + fwd32),
+                                 "fp32_block_marks": 1000.0 / (proj_ms + bin_ms + fwd32m)},
+            "train_step_ms_fp32": proj_ms + bin_ms + fwd32m + bwd_ms + pbwd_ms,
             "train_step_ms_tc_fwd": proj_ms + bin_ms + fwdtc + bwd_ms + pbwd_ms,
             "train_step_note": "forward and backward to the 3D parameters (means, scales, quaternions, opacity, "
                                "SH); per-stage CUDA events with L2 flushed before each stage",
@@ -354,8 +364,8 @@ def bench_differentiation(dev, flush):
 def _sched_run(dev, eval_cams, scene, train_cams, label, chunk=16):
     """Train the tile-cost MLP on the tile costs recorded by renders of train_cams, then time the
     batched render of eval_cams in natural, list-length and MLP order; also the FP32 arms of the same
-    batch: the batched renderer with its product on CUDA cores (list-length order) and the 3DGS-style
-    FP32 kernel launched view by view."""
+    batch: the batched renderer with its product on CUDA cores (list-length order) and the FP32
+    kernel launched view by view, without (the 3DGS baseline) and with its block tests."""
     import torch
     import paper_2505_24796_gb300 as tc
     from oracle import sched as osc
@@ -416,14 +426,14 @@ def _sched_run(dev, eval_cams, scene, train_cams, label, chunk=16):
     t_cc = mv_cc.time_render(q_len, reps=15, warmup=3)
     del mv_cc
 
-    opts32 = tc.render_opts("fp32")
-
-    def per_view_fp32():
+    def per_view_fp32(opts):
         for r in mv.views:
-            tc.tcgs_render_fwd(r.cam, opts32, r.bins["tile_ranges"], r.bins["ids_sorted"], r.proj["mean2d"],
+            tc.tcgs_render_fwd(r.cam, opts, r.bins["tile_ranges"], r.bins["ids_sorted"], r.proj["mean2d"],
                                r.proj["conic"], d["opacity"], r.proj["rgb"], out=r.out)
-    t_fp32 = _events_ms(per_view_fp32, 15, 3)
-    res["fp32_arms_ms"] = {"batched_same_skip_length_order": t_cc, "fp32_3dgs_kernel_view_by_view": t_fp32}
+    t_fp32, t_fp32m = (_events_ms(lambda: per_view_fp32(tc.render_opts("fp32", tile_cull=marks)), 15, 3)
+                       for marks in (False, True))
+    res["fp32_arms_ms"] = {"batched_same_skip_length_order": t_cc, "fp32_3dgs_kernel_view_by_view": t_fp32,
+                           "fp32_block_marks_view_by_view": t_fp32m}
     res["speedup_tc_mlp_vs_fp32"] = {"vs_same_skip_batched": t_cc / times["mlp"], "vs_fp32_view_by_view": t_fp32 / times["mlp"]}
     return res
 
@@ -471,9 +481,9 @@ def bench_large(dev, flush, steps=5, warmup=2):
     shared = [_events_ms(lambda: r.project(d), steps, warmup, flush),
               _events_ms(lambda: r.bin_sort(), steps, warmup, flush)]
     out["shared_stages_note"] = "project and bin_sort timed once (identical for both renderers)"
-    for prec in ("tc_fp16_split", "fp32", "fp32_frag2mat"):
-        stg = shared + [_events_ms(lambda: r.render(d["opacity"], prec), steps, warmup, flush)]
-        out[prec] = {"stages_ms": dict(zip(["project", "bin_sort", "render_fwd"], stg)), "frame_ms": sum(stg),
+    for arm, (prec, kw) in ARMS.items():
+        stg = shared + [_events_ms(lambda: r.render(d["opacity"], prec, **kw), steps, warmup, flush)]
+        out[arm] = {"stages_ms": dict(zip(["project", "bin_sort", "render_fwd"], stg)), "frame_ms": sum(stg),
                      "frames_per_s": 1000.0 / sum(stg)}
     out["speedup_render"] = out["fp32"]["stages_ms"]["render_fwd"] / out["tc_fp16_split"]["stages_ms"]["render_fwd"]
     out["speedup_render_vs_fp32_same_skip"] = (out["fp32_frag2mat"]["stages_ms"]["render_fwd"] /
@@ -517,7 +527,9 @@ def _coverage_render(cam, d, capacity, dev, flush, exact, steps=10, warmup=3):
     out = {"splats": int(r.bins["n_splats"].item()),
            "ms": {"bin_sort": _events_ms(lambda: r.bin_sort(), steps, warmup, flush),
                   "render_fwd_tc": _events_ms(lambda: r.render(d["opacity"], "tc_fp16_split"), steps, warmup, flush),
-                  "render_fwd_fp32": _events_ms(lambda: r.render(d["opacity"], "fp32"), steps, warmup, flush)}}
+                  "render_fwd_fp32": _events_ms(lambda: r.render(d["opacity"], "fp32", tile_cull=False), steps, warmup,
+                                                flush),
+                  "render_fwd_fp32_block_marks": _events_ms(lambda: r.render(d["opacity"], "fp32"), steps, warmup, flush)}}
     del r
     torch.cuda.empty_cache()
     return out
@@ -525,8 +537,9 @@ def _coverage_render(cam, d, capacity, dev, flush, exact, steps=10, warmup=3):
 
 ABLATION = [
     # (label, precision, early_cull, tile_cull): Table 4 (EarlyCull x Frag2Mat with G2L) ...
-    ("fp32", "fp32", False, True),
-    ("fp32+earlycull", "fp32", True, True),
+    ("fp32", "fp32", False, False),   # the 3DGS baseline, and the base of speedup_vs_fp32
+    ("fp32+earlycull", "fp32", True, False),
+    ("fp32+block_marks", "fp32", False, True),
     # the tensor-core renderer with its product u^T v on CUDA cores in FP32: the same schedule, staging,
     # block marks and EarlyCull, so against the rows below only the tensor-core product differs
     ("fp32_frag2mat_g2l+earlycull", "fp32_frag2mat", True, False),
@@ -543,6 +556,11 @@ ABLATION = [
 ]
 
 
+def has_block_marks(precision, tile_cull):
+    """Whether the configuration skips list entries per pixel block."""
+    return bool(tile_cull) and not precision.endswith("_global")
+
+
 def bench_ablation(r, dsc, flush, img32, oracle_img=None, mask=None, reps=10, warmup=3):
     """Render-stage time and accuracy of each configuration of ABLATION on one frame's bins."""
     import torch
@@ -555,7 +573,7 @@ def bench_ablation(r, dsc, flush, img32, oracle_img=None, mask=None, reps=10, wa
         torch.cuda.synchronize()
         im = r.out["img"].cpu().numpy().astype(np.float64)
         row = {"precision": prec, "early_cull": ec,
-               "block_marks": tcull and prec != "fp32" and not prec.endswith("_global"),
+               "block_marks": has_block_marks(prec, tcull),
                "render_ms": ms, "finite": bool(np.isfinite(im).all())}
         mse = float(np.mean((im - ref32) ** 2))
         row["psnr_vs_fp32_db"] = 10 * math.log10(1 / mse) if mse > 0 else None
@@ -571,13 +589,13 @@ def bench_ablation(r, dsc, flush, img32, oracle_img=None, mask=None, reps=10, wa
     return out
 
 
-def time_frames(r, dsc, precision, steps, warmup, use_graph, flush, stream):
+def time_frames(r, dsc, precision, steps, warmup, use_graph, flush, stream, **kw):
     """Frames of renderer r (project -> bin_sort -> render); L2 flushed before every timed frame,
     outside the events.  With graphs, the frame time comes from one CUDA graph holding the whole
     frame (as a renderer would replay it), and the stage times from a second set of steps with one
-    graph per stage and events between them.  Returns the frame times and the per-stage times (ms)."""
+    graph per stage and events between them.  kw: render options.  Returns the frame times and the per-stage times (ms)."""
     import torch
-    fns = [lambda: r.project(dsc), lambda: r.bin_sort(), lambda: r.render(dsc["opacity"], precision)]
+    fns = [lambda: r.project(dsc), lambda: r.bin_sort(), lambda: r.render(dsc["opacity"], precision, **kw)]
     frame = None
     if use_graph:
         for f in fns:
@@ -629,7 +647,7 @@ def time_frames(r, dsc, precision, steps, warmup, use_graph, flush, stream):
     return total, per_stage
 
 
-def time_frames_two_in_flight(renderers, dsc, precision, frames, warmup, flush):
+def time_frames_two_in_flight(renderers, dsc, precision, frames, warmup, flush, **kw):
     """Throughput of a stream of independent frames with two in flight: renderer i (own buffers) replays
     its whole-frame CUDA graph on its own stream, frames alternating between the two, so one frame's
     sort can overlap the other's render.  L2 flushed once before the timed frames.  Returns ms per frame."""
@@ -638,11 +656,11 @@ def time_frames_two_in_flight(renderers, dsc, precision, frames, warmup, flush):
     graphs = []
     for r, st in zip(renderers, streams):
         with torch.cuda.stream(st):
-            r.frame(dsc, precision=precision)
+            r.frame(dsc, precision=precision, **kw)
             torch.cuda.synchronize()
             g = torch.cuda.CUDAGraph()
             with torch.cuda.graph(g, stream=st):
-                r.frame(dsc, precision=precision)
+                r.frame(dsc, precision=precision, **kw)
         graphs.append(g)
     torch.cuda.synchronize()
 
@@ -763,11 +781,15 @@ def run_tcgs(args):
     capacity = n_splats + 1024
     exact = args.coverage == "exact"
     r = tc.Renderer(cam, P, capacity, device=dev, stats=True, exact_tiles=exact)
-    r.frame(dsc, precision="fp32")
-    torch.cuda.synchronize()
+    slots = {}
+    for arm in ("fp32_block_marks", "fp32"):
+        r.stats.zero_()
+        r.frame(dsc, precision=ARMS[arm][0], **ARMS[arm][1])
+        torch.cuda.synchronize()
+        st = r.stats.to(torch.int64).sum(dim=0).tolist()
+        slots[arm] = st[2]
     n_binned = int(r.bins["n_splats"].item())
-    st = r.stats.to(torch.int64).sum(dim=0).tolist()
-    f_blend, f_cull, slots_fp32 = st[0], st[1], st[2]
+    f_blend, f_cull = st[0], st[1]
     alpha_evals = f_blend + f_cull
     img_fp32 = r.out["img"].clone()
     r.stats.zero_()
@@ -782,9 +804,11 @@ def run_tcgs(args):
     stream = torch.cuda.current_stream(dev)
 
     use_graph = not args.no_graph
-    # --- FP32 comparison paths: the 3DGS baseline kernel, and the tensor-core renderer with its product on
-    # CUDA cores (same schedule, block marks and EarlyCull: only the tensor-core product differs)
-    tot32, st32 = time_frames(r, dsc, "fp32", args.steps, args.warmup, use_graph, flush, stream)
+    # --- FP32 comparison paths: the 3DGS baseline kernel, the same with its block tests, and the tensor-core
+    # renderer with its product on CUDA cores (same schedule, block marks and EarlyCull: only the tensor-core
+    # product differs)
+    tot32, st32 = time_frames(r, dsc, "fp32", args.steps, args.warmup, use_graph, flush, stream, tile_cull=False)
+    tot32m, st32m = time_frames(r, dsc, "fp32", args.steps, args.warmup, use_graph, flush, stream, tile_cull=True)
     totcc, stcc = time_frames(r, dsc, "fp32_frag2mat", args.steps, args.warmup, use_graph, flush, stream)
     # --- headline path, with clocks sampled during the timed region; a barrier and a device
     # synchronisation on both sides of it
@@ -810,8 +834,8 @@ def run_tcgs(args):
     # --- two independent frames in flight on two streams (a serving loop's throughput), beside the
     # per-frame figure above
     r2 = tc.Renderer(cam, P, capacity, device=dev, exact_tiles=exact)
-    two_ms = {prec: time_frames_two_in_flight([r, r2], dsc, prec, 4 * args.steps, args.warmup, flush)
-              for prec in (args.precision, "fp32")}
+    two_ms = {prec: time_frames_two_in_flight([r, r2], dsc, prec, 4 * args.steps, args.warmup, flush, **kw)
+              for prec, kw in ((args.precision, {}), ARMS["fp32"])}
     del r2
 
     # --- end to end through the public API with host buffers: every frame's scene goes host -> device
@@ -886,8 +910,8 @@ def run_tcgs(args):
         torch.cuda.synchronize()
         other = {"coverage": "square" if exact else "exact", "splats": int(r_o.bins["n_splats"].item())}
         img_o32 = r_o.out["img"].clone()
-        for prec in (args.precision, "fp32"):
-            tq, sq = time_frames(r_o, dsc, prec, args.steps, args.warmup, use_graph, flush, stream)
+        for prec, kw in ((args.precision, {}), ARMS["fp32"]):
+            tq, sq = time_frames(r_o, dsc, prec, args.steps, args.warmup, use_graph, flush, stream, **kw)
             other[prec] = {"frames_per_s": 1000.0 / statistics.mean(tq),
                            "stages_ms": dict(zip(["project", "bin_sort", "render_fwd"],
                                                  [statistics.mean(x) for x in sq]))}
@@ -986,17 +1010,22 @@ def run_tcgs(args):
         "stages_ms": dict(zip(stage_names, stage_ms)),
         "fp32": {"frames_per_s": 1000.0 / ms32, "ms_per_step": ms32,
                  "stages_ms": dict(zip(stage_names, [statistics.mean(s) for s in st32])),
-                 "alpha_evals_per_s": alpha_evals / (render32_ms * 1e-3)},
+                 "alpha_evals_per_s": alpha_evals / (render32_ms * 1e-3),
+                 "kernel": "k_render_fp32 with tile_cull = 0: every list entry at every pixel (the 3DGS baseline)"},
+        "fp32_block_marks": {"frames_per_s": 1000.0 / statistics.mean(tot32m), "ms_per_step": statistics.mean(tot32m),
+                             "stages_ms": dict(zip(stage_names, [statistics.mean(s) for s in st32m])),
+                             "kernel": "k_render_fp32 with its block tests (tile_cull = 1, the default)"},
         "fp32_same_skip": {"frames_per_s": 1000.0 / statistics.mean(totcc), "ms_per_step": statistics.mean(totcc),
                            "stages_ms": dict(zip(stage_names, [statistics.mean(s) for s in stcc])),
                            "kernel": "k_render_tc with the product u^T v on CUDA cores (TCGS_FP32_FRAG2MAT)"},
         "two_frames_in_flight": {"frames_per_s": {k: 1000.0 / v for k, v in two_ms.items()},
                                  "note": "independent frames alternating between two renderers and two streams, "
                                          "each frame one CUDA graph; the headline value is one frame at a time"},
-        "speedup_vs_fp32": {"frame": ms32 / ms, "render": render32_ms / render_ms,
+        "speedup_vs_fp32": {"base": "fp32 (tile_cull = 0)", "frame": ms32 / ms, "render": render32_ms / render_ms,
+                            "render_vs_block_marks": statistics.mean(st32m[2]) / render_ms,
                             "render_vs_same_skip": statistics.mean(stcc[2]) / render_ms},
         "accuracy": acc, "status": {"bin_sort": status[0], "render": status[1]},
-        "executed_fragment_slots": {"fp32": slots_fp32, "tc": st_tc[2]},
+        "executed_fragment_slots": {**slots, "tc": st_tc[2]},
         "roofline": roof, "roofline_all": {"project": rl_proj, "bin_sort": rl_bin, "render_fwd": rl_render},
         "cpu_baseline": cpu_baseline, "cpu_baseline_all_cores": cpu_all,
         "e2e": {"value": e2e_fps, "unit": "frames/s", "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
@@ -1030,7 +1059,8 @@ def run_large_frames(args):
     r = tc.Renderer(cam, len(sc["opacity"]), n + 1024, device="cuda")
     steps = [("project", lambda: r.project(d)), ("bin_sort", lambda: r.bin_sort()),
              ("render_tc", lambda: r.render(d["opacity"], "tc_fp16_split")),
-             ("render_fp32", lambda: r.render(d["opacity"], "fp32"))]
+             ("render_fp32", lambda: r.render(d["opacity"], "fp32", tile_cull=False)),
+             ("render_fp32_block_marks", lambda: r.render(d["opacity"], "fp32"))]
     for frame in range(2):
         ms = {}
         for name, fn in steps:
@@ -1108,13 +1138,14 @@ def run_render_arms(args):
     torch.cuda.synchronize()
     for rep in range(2):
         ms = {}
-        for prec in ("tc_fp16_split", "fp32_frag2mat", "fp32"):
+        for arm in ("tc_fp16_split", "fp32_frag2mat", "fp32", "fp32_block_marks"):
+            prec, kw = ARMS[arm]
             e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
             e0.record()
-            r.render(d["opacity"], prec)
+            r.render(d["opacity"], prec, **kw)
             e1.record()
             e1.synchronize()
-            ms[prec] = e0.elapsed_time(e1)
+            ms[arm] = e0.elapsed_time(e1)
         print(json.dumps({"render_arms": rep, "splats": int(r.bins["n_splats"].item()), "ms": ms}), flush=True)
 
 
