@@ -105,39 +105,6 @@ __device__ __forceinline__ int clamp_tile(float f, int lo, int hi) {
     return (int)fminf(fmaxf(f, (float)lo), (float)hi);   // NaN -> lo
 }
 
-// The shadow [xa, xb] of the ellipse on the x axis within tile row ty's band [yl, yh] of pixel centres, relative to
-// the mean (in: the band meets the ellipse); rl and rr: half the slope of the form across its ends, at the offsets
-// dl and dr where the ellipse reaches furthest inside the band.
-struct Shadow {
-    float yl, yh, xa, xb, rl, rr;
-    bool in;
-};
-
-__device__ __forceinline__ Shadow shadow_of(const Cover& v, const Reach& e, int ty) {
-    Shadow h;
-    h.yl = __fsub_rn((float)(ty * kTile) + 0.5f, v.my);
-    h.yh = __fadd_rn(h.yl, 15.f);
-    h.xa = h.xb = h.rl = h.rr = 0.f;
-    h.in = !(h.yl > e.H || h.yh < -e.H);
-    if (h.in) {
-        const float alim = __fmul_rn(v.a, v.lim);
-        const float dl = fminf(h.yh, fmaxf(h.yl, e.s)), dr = fminf(h.yh, fmaxf(h.yl, -e.s));
-        h.rl = __fsqrt_rn(fmaxf(0.f, __fsub_rn(alim, __fmul_rn(e.det, __fmul_rn(dl, dl)))));
-        h.rr = __fsqrt_rn(fmaxf(0.f, __fsub_rn(alim, __fmul_rn(e.det, __fmul_rn(dr, dr)))));
-        h.xa = __fmul_rn(__fsub_rn(__fmul_rn(-v.b, dl), h.rl), v.ia);
-        h.xb = __fmul_rn(__fadd_rn(__fmul_rn(-v.b, dr), h.rr), v.ia);
-    }
-    return h;
-}
-
-// First and last tile whose box [16 tx + 0.5, 16 tx + 15.5] meets [mx + xa, mx + xb].
-__device__ __forceinline__ float first_met(const Cover& v, float xa) {
-    return ceilf(__fmul_rn(__fsub_rn(__fadd_rn(v.mx, xa), 15.5f), 1.f / kTile));
-}
-__device__ __forceinline__ float last_met(const Cover& v, float xb) {
-    return floorf(__fmul_rn(__fsub_rn(__fadd_rn(v.mx, xb), 0.5f), 1.f / kTile));
-}
-
 // Tiles [L, R] (empty when L > R) of rectangle columns [x0, x1] in tile row ty that Gaussian v reaches.
 __device__ int2 row_span(const Cover& v, const Reach& e, int ty, int x0, int x1) {
     const int2 none = make_int2(1, 0);
@@ -153,9 +120,22 @@ __device__ int2 row_span(const Cover& v, const Reach& e, int ty, int x0, int x1)
         return make_int2(L, R);
     };
     if (e.W < 0.f || x1 - x0 < 3) return scan();
-    const Shadow h = shadow_of(v, e, ty);
-    const float yl = h.yl, yh = h.yh, xa_ = h.xa, xb_ = h.xb, rl_ = h.rl, rr_ = h.rr;
-    const float Lf = h.in ? first_met(v, xa_) : 1.f, Rf = h.in ? last_met(v, xb_) : 0.f;   // empty unless the band meets the ellipse
+    // the shadow [xa, xb] of the ellipse on the x axis within the row's band of pixel centres
+    const float yl = __fsub_rn((float)(ty * kTile) + 0.5f, v.my), yh = __fadd_rn(yl, 15.f);
+    float Lf = 1.f, Rf = 0.f;   // empty unless the band meets the ellipse
+    float xa_ = 0.f, xb_ = 0.f, rl_ = 0.f, rr_ = 0.f;
+    if (!(yl > e.H || yh < -e.H)) {
+        const float alim = __fmul_rn(v.a, v.lim);
+        const float dl = fminf(yh, fmaxf(yl, e.s)), dr = fminf(yh, fmaxf(yl, -e.s));
+        const float rl = __fsqrt_rn(fmaxf(0.f, __fsub_rn(alim, __fmul_rn(e.det, __fmul_rn(dl, dl)))));
+        const float rr = __fsqrt_rn(fmaxf(0.f, __fsub_rn(alim, __fmul_rn(e.det, __fmul_rn(dr, dr)))));
+        const float xa = __fmul_rn(__fsub_rn(__fmul_rn(-v.b, dl), rl), v.ia);
+        const float xb = __fmul_rn(__fadd_rn(__fmul_rn(-v.b, dr), rr), v.ia);
+        xa_ = xa; xb_ = xb; rl_ = rl; rr_ = rr;
+        // tiles whose box [16 tx + 0.5, 16 tx + 15.5] meets [mx + xa, mx + xb]
+        Lf = ceilf(__fmul_rn(__fsub_rn(__fadd_rn(v.mx, xa), 15.5f), 1.f / kTile));
+        Rf = floorf(__fmul_rn(__fsub_rn(__fadd_rn(v.mx, xb), 0.5f), 1.f / kTile));
+    }
     if (!(Lf <= Rf) || Rf < (float)x0 || Lf > (float)x1) {
         // no shadow in the rectangle: probe the tile holding the point of least q in the band (the
         // least of the minima over x, (det / a) dy^2, is at the dy nearest to 0), grow from there
@@ -203,6 +183,39 @@ __device__ int2 row_span(const Cover& v, const Reach& e, int ty, int x0, int x1)
         R = k;
     }
     return make_int2(L, R);
+}
+
+// The shadow [xa, xb] of the ellipse on the x axis within tile row ty's band [yl, yh] of pixel centres, relative to
+// the mean (in: the band meets the ellipse); rl and rr: half the slope of the form across its ends, at the offsets
+// dl and dr where the ellipse reaches furthest inside the band.  (As row_span forms it.)
+struct Shadow {
+    float yl, yh, xa, xb, rl, rr;
+    bool in;
+};
+
+__device__ __forceinline__ Shadow shadow_of(const Cover& v, const Reach& e, int ty) {
+    Shadow h;
+    h.yl = __fsub_rn((float)(ty * kTile) + 0.5f, v.my);
+    h.yh = __fadd_rn(h.yl, 15.f);
+    h.xa = h.xb = h.rl = h.rr = 0.f;
+    h.in = !(h.yl > e.H || h.yh < -e.H);
+    if (h.in) {
+        const float alim = __fmul_rn(v.a, v.lim);
+        const float dl = fminf(h.yh, fmaxf(h.yl, e.s)), dr = fminf(h.yh, fmaxf(h.yl, -e.s));
+        h.rl = __fsqrt_rn(fmaxf(0.f, __fsub_rn(alim, __fmul_rn(e.det, __fmul_rn(dl, dl)))));
+        h.rr = __fsqrt_rn(fmaxf(0.f, __fsub_rn(alim, __fmul_rn(e.det, __fmul_rn(dr, dr)))));
+        h.xa = __fmul_rn(__fsub_rn(__fmul_rn(-v.b, dl), h.rl), v.ia);
+        h.xb = __fmul_rn(__fadd_rn(__fmul_rn(-v.b, dr), h.rr), v.ia);
+    }
+    return h;
+}
+
+// First and last tile whose box [16 tx + 0.5, 16 tx + 15.5] meets [mx + xa, mx + xb].
+__device__ __forceinline__ float first_met(const Cover& v, float xa) {
+    return ceilf(__fmul_rn(__fsub_rn(__fadd_rn(v.mx, xa), 15.5f), 1.f / kTile));
+}
+__device__ __forceinline__ float last_met(const Cover& v, float xb) {
+    return floorf(__fmul_rn(__fsub_rn(__fadd_rn(v.mx, xb), 0.5f), 1.f / kTile));
 }
 
 // Bound on the relative error of Reach.s: that of the determinant is 1.2e-7 ac / det, of which the ellipse's width

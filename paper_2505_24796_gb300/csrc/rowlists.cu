@@ -31,11 +31,13 @@ constexpr int kRowThreads = 256;             // also the Gaussians of a span blo
 constexpr int kRowWarps = kRowThreads / 32;
 constexpr int kChunk = 512;                  // runs expanded together: 16 words of the bit matrix per column
 constexpr int kChunkWords = kChunk / 32;
+constexpr uint32_t kOneTest = 1u << 16;      // a row to test, beside the runs that a round of spans has so far
 constexpr int kSpanBuffer = 3072;            // runs of a span block kept in shared memory (more: evaluated twice)
 constexpr int kScatterStage = 4096;          // runs regrouped by row at a time
 constexpr int kExpandStage = 3584;           // ids regrouped by column at a time (4 expand blocks an SM up to 256 columns)
 static_assert(kRowThreads == kRowListsMaxGrid && kChunk <= kExpandStage && kRowThreads <= kScatterStage,
               "a thread per row or column; a column of a chunk, or a row of a block, fits the stage");
+static_assert(kRowThreads * (kRowMinWidth / 2) < kOneTest, "the runs of a round's narrow and decided rows");
 
 // Counters zeroed by k_row_keys.
 struct RowCounters {
@@ -104,8 +106,8 @@ __global__ void __launch_bounds__(kRowThreads) k_row_keys(uint32_t P, const floa
     }
 }
 
-// Runs of reached tiles of a wide Gaussian whose row has no closed form that decides it (a conic that is not
-// positive definite, a needle), every tile of columns [x0, x1] of row ty tested: one run from the first to the last reached tile with `fill`, else every
+// Runs of reached tiles of a wide Gaussian whose conic is not positive definite, every tile of columns
+// [x0, x1] of row ty tested: one run from the first to the last reached tile with `fill`, else every
 // maximal run.  Returns their number, adds their length to `len`, and stores those below `most` to
 // dst (null: none).  Out of line: counting and storing then take the same decisions.
 __device__ __noinline__ uint32_t tested_runs(const Cover& v, int ty, int x0, int x1, bool fill, uint32_t head,
@@ -135,12 +137,19 @@ __device__ __noinline__ uint32_t tested_runs(const Cover& v, int ty, int x0, int
 // which keeps the depth order inside every row.  A block reserves its slice of `runs` with one atomic
 // once it knows its size (slices in any order: the offsets find them by block), from shared memory;
 // a block with more than kSpanBuffer runs evaluates them a second time instead.
-// Six blocks an SM (the compiler takes 48 registers for five): runs of the 1920 x 1080 frame 68 -> 64 us, of 605M
-// splats at 3840 x 2160 1.59 -> 1.53 ms.  Rows that no closed form decides to the last tile are tested tile by tile:
-// 20,000 needles of 20 to 300 pixels in 170,000 Gaussians sort in 1.44 ms (in 0.25 ms, with a tile in 10^6 kept or
-// left out otherwise, when their rows' ends alone are tested).
-template <bool EXACT>
-__global__ void __launch_bounds__(kRowThreads, 6) k_row_spans(DevCamera cam, uint32_t P,
+// EXACT: RowLists.exact.  TILES: exact without fill_rows, every tile kept or left out as the per-tile test decides: a wide
+// row is taken from the closed form where that decides every tile of it (row_tiles), else the block's warps test it, 32
+// tiles at a time.  20,000 needles of 20 to 300 pixels in 170,000 Gaussians sort in 0.57 ms (3.55 ms by radix passes
+// that test every tile; 0.25 ms, with a tile in 10^6 kept or left out otherwise, when the rows' ends alone are
+// tested; 1.45 ms with a lane a row, where one needle across the view was the tail of its block).  The 1237 x 701
+// frame takes 4 us more than with the ends alone, the 1920 x 1080 one 1 us.
+// fill_rows is read where it is always set: as a constant it has the compiler contract row_span's tests
+// otherwise, which moves FP32 ties.
+// An instance of its own: in one kernel with row_span both take more registers (605M splats at 3840 x 2160:
+// 1.51 -> 1.59 ms); five blocks an SM, as the other takes by itself (four: 1920 x 1080 6 us slower, 1237 x 701 4
+// us faster).
+template <bool EXACT, bool TILES>
+__global__ void __launch_bounds__(kRowThreads, TILES ? 5 : 0) k_row_spans(DevCamera cam, uint32_t P,
                                                            const uint32_t* __restrict__ order,
                                                            const float* __restrict__ mean2d,
                                                            const int32_t* __restrict__ radius,
@@ -156,6 +165,10 @@ __global__ void __launch_bounds__(kRowThreads, 6) k_row_spans(DevCamera cam, uin
     __shared__ uint32_t s_ws[kRowWarps];
     __shared__ unsigned long long s_len, s_base;
     __shared__ uint32_t s_multi;
+    // TILES: the rows to test, their threads, and each thread's row's bits, [32 tiles][thread]
+    __shared__ uint32_t s_task[TILES ? kRowThreads : 1];
+    __shared__ uint8_t s_thread[TILES ? kRowThreads : 1];
+    extern __shared__ uint32_t s_mask[];
     const int t = threadIdx.x;
     const uint32_t i = blockIdx.x * kRowThreads + t;
     uint32_t rows = 0, rect = 0;
@@ -190,7 +203,7 @@ __global__ void __launch_bounds__(kRowThreads, 6) k_row_spans(DevCamera cam, uin
         for (uint32_t r0 = 0; r0 < total_rows; r0 += kRowThreads) {
             const uint32_t rr = r0 + (uint32_t)t;
             const bool active = rr < total_rows;
-            uint32_t owner = 0, n = 0, len = 0, reached = 0;   // reached: the tiles of at most 32 tested, one bit each
+            uint32_t owner = 0, n = 0, len = 0, reached = 0;   // reached: a narrow row's tiles, one bit each
             int ty = 0, x0 = 0, x1 = 0, L = 0, R = -1;
             bool tested = false;
             if (active) {
@@ -203,34 +216,32 @@ __global__ void __launch_bounds__(kRowThreads, 6) k_row_spans(DevCamera cam, uin
                 ty = (int)((rc >> 16) & 0xFFu) + (int)(rr - s_pre[owner]);
                 if (!EXACT) {
                     L = x0; R = x1;
+                } else if (x1 - x0 + 1 < kRowMinWidth) {   // tile by tile
+                    const Cover& v = s_cv[owner];
+                    const float ly = v.my - (float)(ty * kTile + kTile / 2);
+                    for (int tx = x0; tx <= x1; ++tx)
+                        if (tile_reached(v, v.mx - (float)(tx * kTile + kTile / 2), ly)) reached |= 1u << (tx - x0);
+                    if (reached) {
+                        L = x0 + __ffs(reached) - 1;
+                        R = x0 + 31 - __clz(reached);
+                        len = __popc(reached);
+                        n = __popc(reached & ~(reached << 1));
+                    }
                 } else {
                     const Cover& v = s_cv[owner];
-                    bool bits = x1 - x0 + 1 < kRowMinWidth;   // few tiles: one by one
-                    if (!bits) {
-                        const Reach e = reach_of(v);
-                        tested = e.W < 0.f;   // not positive definite: no closed form
-                        if (!tested && fill_rows) {
-                            const int2 sp = row_span(v, e, ty, x0, x1);
-                            L = sp.x; R = sp.y;
-                        } else if (!tested) {
+                    const Reach e = reach_of(v);
+                    tested = e.W < 0.f;
+                    if constexpr (TILES) {
+                        if (!tested) {
                             const RowTiles q = row_tiles(v, e, turn_error(v), ty, x0, x1);
                             x0 = L = q.lo; x1 = R = q.hi;
-                            bits = !q.sure && x1 - x0 < 32;
-                            tested = !q.sure && !bits;
+                            tested = !q.sure;
                         }
-                        if (tested) n = tested_runs(v, ty, x0, x1, fill_rows != 0, 0u, nullptr, 0u, len);
-                    }
-                    if (bits) {
-                        const float ly = v.my - (float)(ty * kTile + kTile / 2);
-                        for (int tx = x0; tx <= x1; ++tx)
-                            if (tile_reached(v, v.mx - (float)(tx * kTile + kTile / 2), ly)) reached |= 1u << (tx - x0);
-                        L = 1; R = 0;
-                        if (reached) {
-                            L = x0 + __ffs(reached) - 1;
-                            R = x0 + 31 - __clz(reached);
-                            len = __popc(reached);
-                            n = __popc(reached & ~(reached << 1));
-                        }
+                    } else if (tested) {
+                        n = tested_runs(v, ty, x0, x1, fill_rows != 0, 0u, nullptr, 0u, len);
+                    } else {   // positive definite: the row's ends in closed form
+                        const int2 sp = row_span(v, e, ty, x0, x1);
+                        L = sp.x; R = sp.y;
                     }
                 }
                 if (n == 0 && L <= R && !tested) {
@@ -239,7 +250,40 @@ __global__ void __launch_bounds__(kRowThreads, 6) k_row_spans(DevCamera cam, uin
                 }
             }
             uint32_t round_n;
-            const uint32_t at = n_out + block_exclusive_scan<uint32_t, kRowThreads>(n, s_ws, round_n);
+            uint32_t at = block_exclusive_scan<uint32_t, kRowThreads>(TILES && tested ? kOneTest : n, s_ws, round_n);
+            if constexpr (TILES) {
+                if (round_n >= kOneTest) {   // uniform: some rows are to be tested
+                    if (tested) {
+                        s_task[at / kOneTest] = owner | (uint32_t)ty << 8 | (uint32_t)x0 << 16 | (uint32_t)x1 << 24;
+                        s_thread[at / kOneTest] = (uint8_t)t;
+                    }
+                    __syncthreads();
+                    for (uint32_t k = t >> 5; k < round_n / kOneTest; k += kRowWarps) {
+                        const uint32_t job = s_task[k], j = s_thread[k];
+                        const Cover& v = s_cv[job & 0xFFu];
+                        const int end = (int)(job >> 24);
+                        const float ly = v.my - (float)((int)((job >> 8) & 0xFFu) * kTile + kTile / 2);
+                        for (int b0 = (int)((job >> 16) & 0xFFu), q = 0; b0 <= end; b0 += 32, ++q) {
+                            const int tx = b0 + (t & 31);
+                            const uint32_t m = __ballot_sync(
+                                0xffffffffu, tx <= end && tile_reached(v, v.mx - (float)(tx * kTile + kTile / 2), ly));
+                            if ((t & 31) == 0) s_mask[q * kRowThreads + j] = m;
+                        }
+                    }
+                    __syncthreads();
+                    if (tested) {
+                        uint32_t carry = 0u;
+                        for (int q = 0; 32 * q <= x1 - x0; ++q) {
+                            const uint32_t m = s_mask[q * kRowThreads + t];
+                            n += __popc(m & ~(m << 1 | carry));
+                            len += __popc(m);
+                            carry = m >> 31;
+                        }
+                    }
+                    at = block_exclusive_scan<uint32_t, kRowThreads>(n, s_ws, round_n);
+                }
+            }
+            at += n_out;
             const uint32_t head = owner | (uint32_t)ty << 8;
             if (pass == 0) {
                 if (n) atomicAdd(&s_rows[ty], n);
@@ -248,12 +292,40 @@ __global__ void __launch_bounds__(kRowThreads, 6) k_row_spans(DevCamera cam, uin
             }
             uint32_t* dst = pass == 0 ? s_buf + at : w.runs + s_base + at;
             const uint32_t most = pass == 0 ? (at < (uint32_t)kSpanBuffer ? (uint32_t)kSpanBuffer - at : 0u) : n;
-            if (EXACT && tested) {
+            if (TILES && tested) {
+                uint32_t k = 0;
+                int open = -1;   // the run that has begun
+                auto emit = [&](int first, int last) {
+                    if (k < most) dst[k] = head | (uint32_t)first << 16 | (uint32_t)last << 24;
+                    ++k;
+                };
+                for (int b0 = x0, q = 0; b0 <= x1; b0 += 32, ++q) {
+                    uint32_t m = s_mask[q * kRowThreads + t];
+                    if (open >= 0 && !(m & 1u)) {   // it ended with the 32 tiles before
+                        emit(open, b0 - 1);
+                        open = -1;
+                    }
+                    while (m) {
+                        const int f = __ffs(m) - 1;
+                        const uint32_t gap = ~(m >> f);
+                        const int end = f + (gap ? __ffs(gap) - 1 : 32);
+                        const int first = f == 0 && open >= 0 ? open : b0 + f;
+                        if (end == 32) {   // it may go on
+                            open = first;
+                            break;
+                        }
+                        emit(first, b0 + end - 1);
+                        open = -1;
+                        m &= 0xFFFFFFFFu << end;
+                    }
+                }
+                if (open >= 0) emit(open, x1);
+            } else if (EXACT && tested) {
                 tested_runs(s_cv[owner], ty, x0, x1, fill_rows != 0, head, dst, most, len);
             } else if (n == 1) {
                 if (most) dst[0] = head | (uint32_t)L << 16 | (uint32_t)R << 24;
             } else if (EXACT) {
-                for (uint32_t k = 0; k < n; ++k) {   // at most 32 tiles reached in parts
+                for (uint32_t k = 0; k < n; ++k) {   // a narrow row reached in parts
                     const int f = __ffs(reached) - 1, e = __ffs(~(reached >> f)) - 1;
                     if (k < most) dst[k] = head | (uint32_t)(x0 + f) << 16 | (uint32_t)(x0 + f + e - 1) << 24;
                     reached &= ~(((1u << e) - 1u) << f);
@@ -538,7 +610,7 @@ __global__ void __launch_bounds__(kColThreads) k_col_offsets(int grid_w, RowScra
 // own.  The ids are regrouped by column in shared memory (column windows of at most kExpandStage ids)
 // and written out in that order, so that each list's part is one contiguous write.
 // Bound by latency (barriers, shared-memory round trips, the loads of a chunk) at 24 warps an SM, so
-// shared memory is sized by the columns there are (4 blocks an SM, 5 up to 185 columns, instead of 3) and
+// shared memory is sized by the columns there are (4 blocks an SM, 5 up to 176 columns, instead of 3) and
 // the next chunk's runs are loaded while the current one is regrouped (2.3M splats at 1920 x 1080: 37 -> 26 us,
 // 605M at 3840 x 2160: 2.73 -> 2.46 ms).  A run's columns dealt to several lanes, and the sets formed by a
 // prefix XOR of two toggles a run instead of one atomic a column, both measured slower.
@@ -696,8 +768,10 @@ void launch_row_lists(const RowLists& a, cudaStream_t s) {
     const RowScratch w = row_scratch(a.scratch, a.P, a.capacity);
     const uint32_t nb = (a.P + kRowThreads - 1) / kRowThreads;
     const int gw = a.cam.grid_w, gh = a.cam.grid_h;
-    launch_pdl(a.exact ? k_row_spans<true> : k_row_spans<false>, nb, kRowThreads, 0, s, a.cam, a.P, a.order, a.mean2d,
-               a.radius, a.conic, a.opacity, (int)a.fill_rows, (unsigned long long)a.capacity, nb, w);
+    const bool tiles = a.exact && !a.fill_rows;
+    launch_pdl(!a.exact ? k_row_spans<false, false> : tiles ? k_row_spans<true, true> : k_row_spans<true, false>, nb,
+               kRowThreads, tiles ? 4 * kRowThreads * ((gw + 31) / 32) : 0, s, a.cam, a.P, a.order, a.mean2d, a.radius,
+               a.conic, a.opacity, (int)a.fill_rows, (unsigned long long)a.capacity, nb, w);
     launch_pdl(k_row_offsets, gh, kScanThreads, 0, s, nb, (long long)a.capacity, a.n_splats, a.status, w);
     count_launches(2);
     if (a.capacity == 0) return;   // N and the status are settled; there is nothing to place
