@@ -31,6 +31,7 @@ constexpr int kRowThreads = 256;             // also the Gaussians of a span blo
 constexpr int kRowWarps = kRowThreads / 32;
 constexpr int kChunk = 512;                  // runs expanded together: 16 words of the bit matrix per column
 constexpr int kChunkWords = kChunk / 32;
+constexpr uint32_t kFiveBlocksFrom = 10;      // span blocks an SM
 constexpr uint32_t kOneTest = 1u << 16;      // a row to test, beside the runs that a round of spans has so far
 constexpr int kSpanBuffer = 3072;            // runs of a span block kept in shared memory (more: evaluated twice)
 constexpr int kScatterStage = 4096;          // runs regrouped by row at a time
@@ -139,17 +140,19 @@ __device__ __noinline__ uint32_t tested_runs(const Cover& v, int ty, int x0, int
 // a block with more than kSpanBuffer runs evaluates them a second time instead.
 // EXACT: RowLists.exact.  TILES: exact without fill_rows, every tile kept or left out as the per-tile test decides: a wide
 // row is taken from the closed form where that decides every tile of it (row_tiles), else the block's warps test it, 32
-// tiles at a time.  20,000 needles of 20 to 300 pixels in 170,000 Gaussians sort in 0.57 ms (3.55 ms by radix passes
+// tiles at a time.  20,000 needles of 20 to 300 pixels in 170,000 Gaussians sort in 0.40 ms (3.55 ms by radix passes
 // that test every tile; 0.25 ms, with a tile in 10^6 kept or left out otherwise, when the rows' ends alone are
-// tested; 1.45 ms with a lane a row, where one needle across the view was the tail of its block).  The 1237 x 701
-// frame takes 4 us more than with the ends alone, the 1920 x 1080 one 1 us.
+// tested; 1.45 ms with a lane a row, where one needle across the view was the tail of its block).
+// kBlocks: five blocks an SM need 48 registers, where the compiler takes 53 and four: the sorting stage of 211,000
+// Gaussians at 1743 x 1004 is 5% slower with five (a chain's loads are not all in flight), of 1M at 1920 x 1080 3%
+// faster; they meet at about kFiveBlocksFrom blocks an SM.  With the better one the 1237 x 701 and 1920 x 1080 frames
+// take what they take when the ends alone are tested, within 0.5%.
 // fill_rows is read where it is always set: as a constant it has the compiler contract row_span's tests
 // otherwise, which moves FP32 ties.
 // An instance of its own: in one kernel with row_span both take more registers (605M splats at 3840 x 2160:
-// 1.51 -> 1.59 ms); five blocks an SM, as the other takes by itself (four: 1920 x 1080 6 us slower, 1237 x 701 4
-// us faster).
-template <bool EXACT, bool TILES>
-__global__ void __launch_bounds__(kRowThreads, TILES ? 5 : 0) k_row_spans(DevCamera cam, uint32_t P,
+// 1.51 -> 1.59 ms).
+template <bool EXACT, bool TILES, int kBlocks = 0>
+__global__ void __launch_bounds__(kRowThreads, kBlocks) k_row_spans(DevCamera cam, uint32_t P,
                                                            const uint32_t* __restrict__ order,
                                                            const float* __restrict__ mean2d,
                                                            const int32_t* __restrict__ radius,
@@ -769,9 +772,12 @@ void launch_row_lists(const RowLists& a, cudaStream_t s) {
     const uint32_t nb = (a.P + kRowThreads - 1) / kRowThreads;
     const int gw = a.cam.grid_w, gh = a.cam.grid_h;
     const bool tiles = a.exact && !a.fill_rows;
-    launch_pdl(!a.exact ? k_row_spans<false, false> : tiles ? k_row_spans<true, true> : k_row_spans<true, false>, nb,
-               kRowThreads, tiles ? 4 * kRowThreads * ((gw + 31) / 32) : 0, s, a.cam, a.P, a.order, a.mean2d, a.radius,
-               a.conic, a.opacity, (int)a.fill_rows, (unsigned long long)a.capacity, nb, w);
+    DeviceInfo d;
+    const bool five = current_device_info(&d) && nb > kFiveBlocksFrom * (uint32_t)d.sms;
+    auto spans = !a.exact ? k_row_spans<false, false> : a.fill_rows ? k_row_spans<true, false>
+                          : five ? k_row_spans<true, true, 5> : k_row_spans<true, true>;
+    launch_pdl(spans, nb, kRowThreads, tiles ? 4 * kRowThreads * ((gw + 31) / 32) : 0, s, a.cam, a.P, a.order, a.mean2d,
+               a.radius, a.conic, a.opacity, (int)a.fill_rows, (unsigned long long)a.capacity, nb, w);
     launch_pdl(k_row_offsets, gh, kScanThreads, 0, s, nb, (long long)a.capacity, a.n_splats, a.status, w);
     count_launches(2);
     if (a.capacity == 0) return;   // N and the status are settled; there is nothing to place

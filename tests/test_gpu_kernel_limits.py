@@ -118,13 +118,14 @@ def _lists(o, gw, cols):
     return lens, o["ids_sorted"][at]
 
 
+@pytest.mark.parametrize("P,seen", [(500_000, 60_000), (200_000, 20_000)])   # more and fewer than 10 blocks of 256 an SM
 @pytest.mark.parametrize("kind", ["needles", "undilated", "axis", "round"])
-def test_row_lists_of_needles_equal_radix_lists(tc, kind):
+def test_row_lists_of_needles_equal_radix_lists(tc, kind, P, seen):
     """Exact coverage tile by tile (fewer than 32 splats of capacity a Gaussian): a view of 256 tile columns, sorted by
     row lists, keeps the tiles of one of 257, whose radix passes test every tile of every rectangle, also for needles
     whose conic form cancels and whose rows are reached in parts."""
     rng = np.random.default_rng(len(kind))
-    P, seen, H = 500_000, 60_000, 1024
+    H = 1024
     L = np.exp(rng.uniform(*np.log([20, 60] if kind == "round" else [100, 1500]), seen))
     s = dict(needles=rng.uniform(0.3, 2, seen), undilated=rng.uniform(1e-3, 0.2, seen), axis=rng.uniform(0.3, 2, seen),
              round=0.8 * L)[kind]
