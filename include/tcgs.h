@@ -229,7 +229,8 @@ TCGS_API tcgs_status tcgs_bin_sort(const tcgs_camera* cam /* host */, int32_t P,
  * minima).  A dropped splat is culled at every pixel of its tile by Algorithm 1, and the margins make
  * that hold for the FP32 and tensor-core renderers' own arithmetic too, so every image rendered from
  * these lists equals the image rendered from tcgs_bin_sort's (only list positions, and so
- * n_contrib, differ).  Order, ranges, outputs, workspace and status as tcgs_bin_sort.
+ * n_contrib, differ).  With splat_capacity >= 32 P the tiles of a wide Gaussian in one row of tiles are kept from
+ * the first to the last reached (the same tiles up to FP32 ties at the limit), else one by one.  Order, ranges, outputs, workspace and status as tcgs_bin_sort.
  * When splat_capacity >= 32 P (wide footprints), Gaussians whose rectangle is at least 6 tiles wide
  * are covered row by row: in a tile row the reached tiles form one run (the region q <= L is
  * convex), found from the ellipse's extent with its end tiles settled by the test above, so the

@@ -1,14 +1,17 @@
 // binsort.cu -- sorting stage (Sec. 3.1, Eq. 3): splats, per-tile depth order, tile ranges.
 //
+// Views of at most 256 x 256 tiles take step 1 and then the row lists of rowlists.cu; small views are ranked by
+// counting and sorted by tile in one CTA; grids beyond 256 columns or rows take all five steps.
+//
 // The paper orders splats by a radix sort of (tile, depth) keys.  We run the same LSD
 // radix sort but hoist its depth digits in front of the duplication:
 //   1. depth keys of the P Gaussians, stable LSD radix sort (4 passes of 8 bits) -> order;
 //   2. exclusive scan of the tile counts in that order -> splat offsets, N, capacity check;
 //   3. duplication in depth order: splat = (tile id, Gaussian id);
-//   4. stable LSD radix sort of the splats by tile id (ceil(log2 tiles / 8) passes);
+//   4. stable LSD radix sort of the splats by tile id (ceil(log2 tiles / 8) passes: 2 or 3);
 //   5. tile ranges from adjacent tile-id changes.
 // Because every pass is stable and duplication preserves the depth order, the result is the
-// (tile, depth, id) order of the 64-bit-key sort, while only 1-2 passes touch the N splats.
+// (tile, depth, id) order of the 64-bit-key sort, while only 2-3 passes touch the N splats.
 // With two tile passes whose high tile bits and Gaussian id fit one 32-bit word together, the first
 // pass writes that word alone, the second sorts the words and writes the ids, and the ranges come
 // from per-tile counts taken in the second pass's histogram (the low tile byte of a position is its
@@ -1073,7 +1076,8 @@ tcgs_status bin_sort(const tcgs_camera* cam, int32_t P, const float* mean2d, con
 
     const bool small = P <= kSmallMaxP && splat_capacity <= kSmallMaxCapacity && num_tiles <= kSmallMaxTiles;
     // the coverage of wide Gaussians by rows pays off for wide footprints: chosen when the caller's capacity
-    // allows at least kRowsCapacityPerGaussian splats per Gaussian (the lists are the same either way)
+    // allows at least kRowsCapacityPerGaussian splats per Gaussian (the lists are the same either way up to FP32 ties
+    // at the reach limit); the row lists keep such rows from their first to their last tile
     const bool rows = exact && splat_capacity >= (int64_t)kRowsCapacityPerGaussian * P;
     if (!small && P > 0 && dc.grid_w <= kRowListsMaxGrid && dc.grid_h <= kRowListsMaxGrid) {
         // depth order, then lists by tile rows (in the workspace from the counts on: the depth passes'
